@@ -65,6 +65,26 @@ def test_importance_and_mask(mc, L, H, nh, frac):
         np.testing.assert_array_equal(mask, ref_mask)
 
 
+@pytest.mark.parametrize("L,H,shift", [(130, 64, 0), (132, 66, 1), (257, 72, 1), (8192, 64, 0), (8193, 64, 0)])
+def test_load_widths_and_mask_kernels(mc, L, H, shift):
+    """Map rows of every alignment (L % 4, a map one float off), token rows that take
+    16-byte loads and ones that do not, NaN above the diagonal (never read into a sum),
+    and the mask on both sides of the rank kernel's limit."""
+    g = torch.Generator(device="cuda").manual_seed(700 + L)
+    buf = torch.rand(L * L + shift, generator=g, device="cuda")
+    attn = buf[shift:].view(1, L, L)
+    above = torch.ones(L, L, dtype=torch.bool, device="cuda").triu(1)
+    attn[0].masked_fill_(above, float("nan"))
+    t = torch.randn(L * H + shift, generator=g, device="cuda").bfloat16()[shift:].view(L, H)
+    imp, mask = mc.token_importance(t, attn, 0.1)
+    col = attn[0].masked_fill(above, 0.0).double().sum(0)
+    ref = t.double().abs().sum(1) * col / torch.arange(L, 0, -1, device="cuda")
+    # fp32 adds of at most 16 rows per partial, H / 32 elements per lane of the l1 norm
+    torch.testing.assert_close(imp.double(), ref, rtol=2e-5, atol=1e-30)
+    n = int(np.ceil(float(np.float32(0.1)) * L - 1e-6))
+    np.testing.assert_array_equal(mask.cpu().numpy(), oracle.select_top(imp.cpu().numpy(), n))
+
+
 def test_mask_ties_go_to_lower_indices(mc):
     """One-hot attention on key 0: every other token has importance 0, so the mask
     is token 0 then the lowest indices."""
