@@ -286,6 +286,7 @@ int mc::moe_forward_ex(const void *x, const void *gate_w, int T, const mc_shape 
     ep.group = shape->group;
     ep.chunks = ws.chunks;
     ep.nchunks = ws.nchunks;
+    ep.offsets = ws.offsets;
     ep.counters = ws.counters;
     ep.x = (const __nv_bfloat16 *)x;
     ep.perm = ws.perm;

@@ -7,32 +7,39 @@
 //   K-major SW128 image the MMA reads (rows = pairs, zero rows past the block),
 //   with the columns of every K = 16 slice ordered like the A operand below.
 // gemm_kernel<W13>: persistent, one CTA per SM, warp-specialised:
-//   producer warp      claims items (a token block x a 128-row block of W1|W3,
-//                      or x a 256-row block pair of W2)
-//                      from an atomic counter and streams per 128-column step
-//                      one ring stage [activation image][packed weights of both
-//                      streams] with cp.async.bulk (half the image for a block of
-//                      <= 64 pairs: the MMA reads rows 0..63 only);
-//   converter warps    two groups of four, taking alternate stages (ping-pong):
-//                      while one group converts its stage, the other's
-//                      tensor-memory stores and barrier waits proceed.  Each warp
-//                      turns its four 16-row tiles (two row tiles x two streams)
-//                      of packed codes (the decode path's layout) into fp16
-//                      (q - z) s and stores them into the group's A buffer in
-//                      tensor memory with tcgen05.st 16x256b, whose thread ->
-//                      (lane, column) order is the mma fragment order the packed
-//                      tiles are stored in;
-//   MMA warps (2)      one per weight stream: tcgen05.mma kind::f16, M = 128
-//                      rows, N = 128 pairs (64 for a block of <= 64 pairs),
-//                      K = 16, A from tensor memory, B from the image, fp32
-//                      accumulators in tensor memory; a stage is issued once its
-//                      converter group has stored it (the group saw the copies
-//                      land), so the MMA warps wait on one barrier per stage;
-//   epilogue warps 4-7 W13: h = silu(W1 x) * (W3 x) -> fp16 image of W2's input
+//   weight producer    claims items (a token block x a 128-row block of W1|W3,
+//                      or x a 256-row block pair of W2) from an atomic counter and
+//                      streams the packed weights of both streams, one 128-column
+//                      step per slot of the weight ring;
+//   image producer     streams the activation images of the same items into a ring
+//                      of its own (only the block's rows, rounded up to 16);
+//   converter warps    16: four for each weight stream and step parity; each warp
+//                      reads its two 16-row tiles of packed codes (the decode path's
+//                      layout) into registers, gives the weight slot back, turns them
+//                      into fp16 (q - z) s, waits until the MMAs have read its A
+//                      buffer two steps ago and stores the tiles there with
+//                      tcgen05.st 16x256b, whose thread -> (lane, column) order is the
+//                      mma fragment order the packed tiles are stored in;
+//   MMA warps (2)      one per weight stream: tcgen05.mma kind::f16, M = 128 rows,
+//                      N = the block's pairs (rounded up to 16), K = 16, A from
+//                      tensor memory, B from the image, fp32 accumulators in tensor
+//                      memory;
+//   epilogue warps     W13: h = silu(W1 x) * (W3 x) -> fp16 image of W2's input
 //                      (the same image layout, one 128-column step per row block);
 //                      W2: fp32 outputs per pair.
-// Tensor memory (512 columns): accumulators of streams 0/1 at columns 0 / 128,
-// the two groups' A buffers of 2 x 64 columns at 256 / 384.
+// What sets the pace.  The tensor pipe takes 1026 cycles for a step's 16 MMAs at
+// N = 128 and 515 at N = 64, whatever copies, tensor-memory stores and shared-memory
+// loads run beside it; the conversion alone takes ~51 cycles per 16x128 tile and SM
+// (820 a step) with 8 warps as with 16: its LOP3, HADD2 and HFMA2 each issue every
+// other cycle.  What kept the MMAs from either pace was their issue: from a
+// `lane == 0` branch 8 MMAs take 541 cycles of moves into uniform registers, and 859
+// beside 16 busy warps (elect_one).  Mixtral-8x7b layer, W1,W3 / W2 launch: 256 tokens
+// (N ~ 60) 157 / 99 -> 135 / 78 us, 4096 tokens 1424 / 755 -> 1298 / 646 us (1.49
+// PFLOP/s, 0.85 of the sustained cuBLAS rate; power-capped).
+// Tensor memory (512 columns): accumulators of streams 0/1 at columns 0 / 128 (when
+// every token block has <= 64 pairs, two accumulator sets of 64 columns each, so
+// that an item's epilogue overlaps the next item's MMAs), each stream's two A
+// buffers of 64 columns at 256 / 384.
 #include "mc_host.h"
 #include "mc_kernels.h"
 #include "mc_profile.h"
@@ -40,59 +47,89 @@
 
 namespace mc {
 
-constexpr int kGN = 128;                  // pairs per token block (MMA N)
+constexpr int kGN = 128;                  // pairs per token block (MMA N), at most
+constexpr int kGNarrow = 64;              // a call whose blocks all have <= 64 pairs: narrow rings
 constexpr int kImgBytes = kGN * kTileK * 2;  // one 128-column step image: 32 KB
-constexpr int kGWBytes = 2 * 8 * (256 * 3 + 128);  // weights of both streams, 3-bit, group 64
-constexpr int kGStage = kImgBytes + kGWBytes;      // 47104 = 46 KB (1024-aligned stages)
-constexpr int kGSlots = 4;
-constexpr int kGHdr = 1024;
-constexpr int kGStaging = kImgBytes;               // epilogue staging of one h image
-constexpr size_t kGSmem = kGHdr + (size_t)kGSlots * kGStage + kGStaging;
-// warps 0-3 / 8-11: converter groups 0 / 1 (warp w: tensor-memory lanes 32 (w % 4)
-// .. +31, tiles 2 (w % 4) and 2 (w % 4) + 1 of each stream); 4-7 epilogue;
-// 12 producer; 13 / 14 issue the MMAs of stream 0 / 1
-constexpr int kGEpi0 = 4, kGProd = 12, kGMma = 13, kGMmaN = 2, kGConvGroup = 4;
-constexpr int kGThreads = 15 * 32;
-constexpr int kGRuns = kMaxE;
-constexpr int kGItemRing = 8;
-constexpr int kGNarrow = 64;                       // blocks of <= 64 pairs: N = 64 MMAs
-static_assert(kGStage % 1024 == 0, "stage alignment");
+constexpr int kGHdr = 2048;
+constexpr size_t kGSmem = 232448;            // all of the CTA's shared memory
+// warps 0-15: converters (warp w: tensor-memory lanes 32 (w % 4) .. +31, i.e. tiles
+// 2 (w % 4) and 2 (w % 4) + 1, of stream (w / 4) % 2, in the steps of parity w / 8);
+// 16-19 epilogue; 20 weight producer; 21 / 22 issue the MMAs of stream 0 / 1; 23
+// image producer
+constexpr int kGConv = 16, kGEpi0 = 16, kGProd = 20, kGMma = 21, kGMmaN = 2, kGImgProd = 23, kGConvGroup = 4;
+constexpr int kGThreads = 24 * 32;
+constexpr int kGMaxW = 8, kGMaxI = 6;        // ring slots, at most
+// Items whose description may still be read while a new one is written: the weight
+// producer is at most kGMaxW + 4 steps (so as many items, at one step per item)
+// ahead of a completed MMA, the epilogue two items behind it, the end marker one
+// more ahead.
+constexpr int kGItemRing = 16;
+static_assert(kGItemRing >= kGMaxW + 4 + 3, "item ring");
+
+// Ring geometry of a call: the weight slots hold a 3-bit step of both streams, the
+// image slots 128 or (narrow) 64 rows; what is left beside the h staging is split so
+// that either ring covers a copy's latency.
+struct GGeom {
+    int atom;               // bytes between an image slot's two 64-column atoms
+    int wslot, nw, ni;      // weight slot bytes, weight and image slots
+    int img0, w0;           // offsets of the rings; the staging starts at kGHdr
+};
+__host__ __device__ __forceinline__ GGeom gemm_geom(int group, bool narrow)
+{
+    GGeom g;
+    g.atom = (narrow ? kGNarrow : kGN) * 128;
+    g.wslot = 2 * supertile_bytes(3, group);
+    g.ni = narrow ? 6 : 4;
+    g.img0 = kGHdr + 2 * g.atom;  // the staging: one h image
+    g.w0 = g.img0 + g.ni * 2 * g.atom;
+    const int nw = ((int)kGSmem - g.w0) / g.wslot;
+    g.nw = nw < kGMaxW ? nw : kGMaxW;
+    return g;
+}
 
 // Byte offset of (pair row n, column c of the 128-column step) in an image: two
 // 64-column SW128 atoms; inside an atom the four 4-column groups of every
 // 16-column run are transposed with the four K = 16 slices, so that K slice s of
 // atom a holds, in order, columns 64a + 16t + 4s + {0..3} for t = 0..3 -- the
 // columns the converter stores into tensor-memory columns 2t / 2t+1 of slice s.
-__host__ __device__ __forceinline__ uint32_t img_off(int n, int c)
+__host__ __device__ __forceinline__ uint32_t img_off(int n, int c, int atom = kGN * 128)
 {
     const int a = c >> 6, cc = c & 63;
     const int t = cc >> 4, s = (cc >> 2) & 3, e = cc & 3;
-    return (uint32_t)a * 16384u + sw128_offset((uint32_t)n, (uint32_t)(16 * s + 4 * t + e));
+    return (uint32_t)(a * atom) + sw128_offset((uint32_t)n, (uint32_t)(16 * s + 4 * t + e));
 }
 
-struct GStage {
-    int item, kt, first, last;  // item id, column step, first / last step of the item
-    int k, u;                   // token block, unit (row block or row-block pair)
-    int narrow;                 // the block has <= 64 pairs
-    ChunkInfo ci;
+// One step of the weight ring (item < 0: end of the CTA's work).
+struct GWStage {
+    int item, bits, nstream, info;  // info: the MMA warps' word (kInfo*)
 };
+constexpr int kInfoN = 0xff, kInfoFirst = 0x100, kInfoLast = 0x200, kInfoLone = 0x400,
+              kInfoEnd = 0x800;
 
 struct GItem {
-    int k, u;  // token block, unit
-    ChunkInfo ci;
+    int k, u, nstream, n;  // token block (-1: end), unit, streams, MMA N
+    int pair_base, nv;
+};
+
+// An expert's token blocks, in the order the items are taken (more bits first).
+struct GRun {
+    int e, bits, off, cnt, first, nb, base;  // expert, its pairs, first block, blocks, first item
 };
 
 struct GShared {
-    uint64_t full[kGSlots], empty[kGSlots];
-    uint64_t afull[2], aempty[2];
-    uint64_t dfull, dempty, esync, drain;
+    uint64_t wfull[kGMaxW], wempty[kGMaxW];
+    uint64_t ifull[kGMaxI], iempty[kGMaxI];
+    uint64_t afull[2][2], aempty[2][2];  // [stream][buffer]
+    uint64_t dfull[2], dempty[2], esync, drain;
+    uint64_t itembar[kGItemRing];
     uint32_t tmem_base;
     volatile int abort;
-    volatile int issued;
+    volatile int wissued, iissued;
     volatile int end_items;  // items this CTA's MMA warps completed, set once they saw the end marker
-    int nruns;
-    int run_first[kGRuns], run_nb[kGRuns], run_base[kGRuns + 1];
-    GStage stage[kGSlots];
+    int total, narrow;
+    int ainfo[2][2];         // [stream][buffer]: the stored step's info word
+    GRun run[kMaxE];
+    GWStage wst[kGMaxW];
     GItem items[kGItemRing];
 };
 static_assert(sizeof(GShared) <= kGHdr, "gemm header");
@@ -110,6 +147,12 @@ __device__ __forceinline__ bool g_wait(uint64_t *bar, uint32_t parity, const Exp
             return false;
         }
     }
+}
+
+// The same for a whole warp, with one answer for all of its lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, const ExpertParams &p, GShared *sh)
+{
+    return __all_sync(0xffffffffu, g_wait(bar, parity, p, sh));
 }
 
 // The packed buffer carries the header written for this shape and bit table
@@ -184,27 +227,39 @@ __device__ __forceinline__ uint32_t pair_offset_bits(int j)
 __device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t *>(&v); }
 __device__ __forceinline__ __half2 bits_h2(uint32_t v) { return *reinterpret_cast<const __half2 *>(&v); }
 
+// The code words and (scale, zero) pairs of one lane's part of a tile, as stored.
+template <int GPT>
+struct RawTile {
+    uint32_t w[6];
+    uint2 meta[GPT];
+};
+
+template <int GPT>
+__device__ __forceinline__ void load_raw(const uint8_t *tile, int bits, int lane, RawTile<GPT> &t)
+{
+    if (bits >= 2) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(tile + 16 * lane);
+        t.w[0] = v.x; t.w[1] = v.y; t.w[2] = v.z; t.w[3] = v.w;
+    }
+    if (bits != 2) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(tile + (bits == 3 ? 512 : 0) + 8 * lane);
+        t.w[4] = v.x; t.w[5] = v.y;
+    }
+    const uint8_t *mt = tile + tile_code_bytes(bits);
+#pragma unroll
+    for (int g = 0; g < GPT; ++g) t.meta[g] = *reinterpret_cast<const uint2 *>(mt + 64 * g + (lane >> 2) * 8);
+}
+
 // One 16-row tile, one 128-column step: 32 fp16 pairs (q - z) s per lane, in the
 // order tcgen05.st 16x256b.x8 takes them: per k-step s, the A-fragment registers
 // a0, a2, a1, a3 (rows g8 / g8+8, k pairs t / t+4).
 template <int BITS, int GPT>
-__device__ __forceinline__ void convert_tile(const uint8_t *tile, int lane, uint32_t (&out)[32])
+__device__ __forceinline__ void convert_tile(const RawTile<GPT> &t, uint32_t (&out)[32])
 {
-    uint32_t c2[4] = {0, 0, 0, 0}, c1[2] = {0, 0};
-    if (BITS >= 2) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(tile + 16 * lane);
-        c2[0] = v.x; c2[1] = v.y; c2[2] = v.z; c2[3] = v.w;
-    }
-    if (BITS != 2) {
-        const uint2 v = *reinterpret_cast<const uint2 *>(tile + (BITS == 3 ? 512 : 0) + 8 * lane);
-        c1[0] = v.x; c1[1] = v.y;
-    }
-    const uint8_t *mt = tile + tile_code_bytes(BITS);
     __half2 s2[GPT][2], nz2[GPT][2];  // [group][row half]: (s, s) and (-z s, -z s)
 #pragma unroll
     for (int g = 0; g < GPT; ++g) {
-        const uint2 m = *reinterpret_cast<const uint2 *>(mt + 64 * g + (lane >> 2) * 8);
-        const __half2 a = bits_h2(m.x), b = bits_h2(m.y);  // (s0, z0), (s1, z1)
+        const __half2 a = bits_h2(t.meta[g].x), b = bits_h2(t.meta[g].y);  // (s0, z0), (s1, z1)
         const float sa = __low2float(a), za = __high2float(a), sb = __low2float(b), zb = __high2float(b);
         s2[g][0] = __floats2half2_rn(sa, sa);
         s2[g][1] = __floats2half2_rn(sb, sb);
@@ -214,12 +269,9 @@ __device__ __forceinline__ void convert_tile(const uint8_t *tile, int lane, uint
 #pragma unroll
     for (int qd = 0; qd < 4; ++qd) {
         uint32_t r[8];
-        if (BITS == 1) cvt1_half(c1[qd >> 1], 8 * (qd & 1), r);
-        if (BITS == 2) cvt2(c2[qd], r);
-        if (BITS == 3) {
-            const uint32_t w[6] = {c2[0], c2[1], c2[2], c2[3], c1[0], c1[1]};
-            cvt3(w, qd, r);
-        }
+        if (BITS == 1) cvt1_half(t.w[4 + (qd >> 1)], 8 * (qd & 1), r);
+        if (BITS == 2) cvt2(t.w[qd], r);
+        if (BITS == 3) cvt3(t.w, qd, r);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = 8 * qd + i, s = j >> 2, rho = j & 3;
@@ -246,11 +298,11 @@ __device__ __forceinline__ void tmem_st_16x256_x8(uint32_t taddr, const uint32_t
 }
 
 template <int GPT>
-__device__ __forceinline__ void convert_regs(const uint8_t *tile, int bits, int lane, uint32_t (&v)[32])
+__device__ __forceinline__ void convert_regs(const RawTile<GPT> &t, int bits, uint32_t (&v)[32])
 {
-    if (bits == 1) convert_tile<1, GPT>(tile, lane, v);
-    else if (bits == 2) convert_tile<2, GPT>(tile, lane, v);
-    else convert_tile<3, GPT>(tile, lane, v);
+    if (bits == 1) convert_tile<1, GPT>(t, v);
+    else if (bits == 2) convert_tile<2, GPT>(t, v);
+    else convert_tile<3, GPT>(t, v);
 }
 
 // ------------------------------------------------------------- epilogue --
@@ -289,341 +341,401 @@ __device__ __forceinline__ bool epi_sync(const ExpertParams &p, GShared *sh, int
 
 // ------------------------------------------------------------------ kernel --
 
-// One converter warp, one stage: its four tiles (tiles 2q, 2q+1 of each stream
-// present), dequantised and stored into A buffer `abuf`; the first store waits
-// until the MMAs that last read the buffer are done (need_wait).  False once the
-// CTA aborted.
-template <int GPT>
-__device__ __forceinline__ bool convert_stage(const uint8_t *w, int bits, int nstream, int STB, int TB, int q,
-                                              int lane, uint32_t abuf, bool need_wait, uint64_t *aempty,
-                                              uint32_t parity, const ExpertParams &p, GShared *sh)
-{
-    uint32_t va[32], vb[32];
-    // two register sets alternate, so that a tile's dequantisation overlaps the
-    // previous tile's store
-    convert_regs<GPT>(w + (2 * q) * TB, bits, lane, va);
-    if (need_wait && !g_wait(aempty, parity, p, sh)) return false;
-    tc_fence_after();
-    tmem_st_16x256_x8(abuf + ((uint32_t)(32 * q) << 16), va);
-    convert_regs<GPT>(w + (2 * q + 1) * TB, bits, lane, vb);
-    tmem_st_16x256_x8(abuf + ((uint32_t)(32 * q + 16) << 16), vb);
-    if (nstream > 1) {
-        convert_regs<GPT>(w + STB + (2 * q) * TB, bits, lane, va);
-        tmem_st_16x256_x8(abuf + 64u + ((uint32_t)(32 * q) << 16), va);
-        convert_regs<GPT>(w + STB + (2 * q + 1) * TB, bits, lane, vb);
-        tmem_st_16x256_x8(abuf + 64u + ((uint32_t)(32 * q + 16) << 16), vb);
-    }
-    tmem_st_wait();
-    return true;
-}
-
 template <bool W13, int GPT>
 __global__ void __launch_bounds__(kGThreads, 1) gemm_kernel(ExpertParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     GShared *sh = reinterpret_cast<GShared *>(smem);
-    uint8_t *ring = smem + kGHdr;
-    uint8_t *staging = smem + kGHdr + (size_t)kGSlots * kGStage;
+    uint8_t *staging = smem + kGHdr;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int group = kTileK / GPT;
+    constexpr int group = kTileK / GPT;
     const int nrb = W13 ? p.F / kBlockRows : p.H / kBlockRows;
     const int KTm = W13 ? p.H / kTileK : p.F / kTileK;  // column steps (K)
     const int U = W13 ? nrb : (nrb + 1) / 2;            // units of a token block: row block (pair)
     const uint8_t *img_base = W13 ? p.ximg : p.himg;
 
-    pdl_wait();
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kGSlots; ++s) {
-            mbar_init(&sh->full[s], 1);
-            mbar_init(&sh->empty[s], kGMmaN + kGConvGroup);  // MMA commits + the stage's converter group
+        for (int s = 0; s < kGMaxW; ++s) {
+            mbar_init(&sh->wfull[s], 1);
+            mbar_init(&sh->wempty[s], 2 * kGConvGroup);
+        }
+        for (int s = 0; s < kGMaxI; ++s) {
+            mbar_init(&sh->ifull[s], 1);
+            mbar_init(&sh->iempty[s], kGMmaN);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&sh->afull[b], kGConvGroup);
-            mbar_init(&sh->aempty[b], kGMmaN);
+            for (int c = 0; c < 2; ++c) {
+                mbar_init(&sh->afull[c][b], kGConvGroup);
+                mbar_init(&sh->aempty[c][b], 1);
+            }
+            mbar_init(&sh->dfull[b], kGMmaN);
+            mbar_init(&sh->dempty[b], 4);
         }
-        mbar_init(&sh->dfull, kGMmaN);
-        mbar_init(&sh->dempty, 4);
         mbar_init(&sh->esync, 4);
         mbar_init(&sh->drain, kGMmaN);
+        for (int i = 0; i < kGItemRing; ++i) mbar_init(&sh->itembar[i], 1);
         sh->abort = 0;
-        sh->issued = 0;
+        sh->wissued = 0;
+        sh->iissued = 0;
         sh->end_items = 0x7fffffff;
-        // runs of token blocks per expert (the block list is grouped by expert)
-        const int nb = *p.nchunks;
-        int r = 0, base = 0;
-        for (int k = 0; k < nb; ++k) {
-            if (k == 0 || p.chunks[k].e != p.chunks[k - 1].e) {
-                if (r > 0) base += sh->run_nb[r - 1] * U;
-                sh->run_first[r] = k;
-                sh->run_nb[r] = 0;
-                sh->run_base[r] = base;
-                ++r;
-            }
-            sh->run_nb[r - 1]++;
-        }
-        sh->nruns = r;
-        sh->run_base[r] = r > 0 ? base + sh->run_nb[r - 1] * U : 0;
         fence_mbar_init();
     }
     if (warp == kGMma) tmem_alloc(&sh->tmem_base, 512);
+    pdl_wait();
+    if (warp == 0) {
+        // the experts' runs of token blocks, from the routing's offsets, in the order
+        // of the block list: more bits first, then by expert
+        const int E = p.E;
+        int off = 0, cnt = 0, bits = 0;
+#pragma unroll
+        for (int f = 0; f < kMaxE; ++f)
+            if (f == lane) bits = p.bits[f];
+        if (lane < E) {
+            off = __ldcg(p.offsets + lane);
+            cnt = __ldcg(p.offsets + lane + 1) - off;
+        }
+        const int nb = (cnt + kGN - 1) / kGN;
+        int rank = 0, first = 0, blocks = 0;
+        for (int f = 0; f < E; ++f) {
+            const int bf = __shfl_sync(0xffffffffu, bits, f), nf = __shfl_sync(0xffffffffu, nb, f);
+            blocks += nf;
+            if (bf > bits || (bf == bits && f < lane)) {
+                ++rank;
+                first += nf;
+            }
+        }
+        if (lane < E) sh->run[rank] = GRun{lane, bits, off, cnt, first, nb, first * U};
+        const unsigned wide = __ballot_sync(0xffffffffu, cnt > kGNarrow);
+        if (lane == 0) {
+            sh->total = blocks * U;
+            sh->narrow = wide == 0;
+        }
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tbase = sh->tmem_base;
-    const int total = sh->run_base[sh->nruns];
+    const int total = sh->total;
+    const bool narrow = sh->narrow;
+    const GGeom geo = gemm_geom(group, narrow);
+    const int nbuf = narrow ? 2 : 1;  // accumulator sets
 
     if (warp == kGProd) {
-        // ------------------------------------------------------------ producer --
+        // ----------------------------------------------------- weight producer --
         if (lane == 0 && !(p.debug & kDebugNoProducer)) {
             const uint64_t pol = policy_evict_first();
-            int it = 0, nitem = 0;
+            int *counter = &p.counters[W13 ? 2 : 3];
             // The packed header was checked once for the call by x_img_kernel, which
             // completed before this launch's wait returned: no copy unless its verdict
-            // says the buffer matches (the verdict's load and the first claim go out
-            // together; the verdict is looked at once the claim returns)
+            // says the buffer matches
             const int verdict = __ldcg(p.hdr_ok);
-            bool ok = true, checked = false;
-            while (ok) {
-                const int item = atomicAdd(&p.counters[W13 ? 2 : 3], 1);
-                if (!checked) {
-                    checked = true;
-                    if (verdict != 1) {
-                        set_status(p.status, MC_ERR_BAD_PACK);
-                        sh->abort = 1;
-                        ok = false;
-                        break;
-                    }
-                }
-                if (item >= total) {
-                    pdl_trigger();  // the CTA takes no further item: the next kernel may launch
-                    break;
-                }
+            int item = atomicAdd(counter, 1);
+            bool ok = verdict == 1;
+            if (!ok) {
+                set_status(p.status, MC_ERR_BAD_PACK);
+                sh->abort = 1;
+            }
+            int it = 0, slot = 0, nitem = 0;
+            uint32_t phase = 0;
+            while (ok && item < total) {
                 int r = 0;
-                while (r + 1 < sh->nruns && item >= sh->run_base[r + 1]) ++r;
-                const int local = item - sh->run_base[r], nbr = sh->run_nb[r];
+                while (r + 1 < p.E && item >= sh->run[r + 1].base) ++r;
+                const GRun run = sh->run[r];
+                const int local = item - run.base;
                 // W1,W3: the expert's token blocks vary fastest, so the CTAs that run
                 // at the same time share a row block's weights (and the blocks' x
                 // images stay in L2); W2: the 256-row block pairs vary fastest, so
                 // they share one block's h image while the expert's W2 weights stay
                 // in L2 from block to block
-                const int u = W13 ? local / nbr : local % U;
-                const int k = sh->run_first[r] + (W13 ? local % nbr : local / U);
-                const ChunkInfo ci = p.chunks[k];
-                const int e = ci.e, bits = ci.bits;
+                const int u = W13 ? local / run.nb : local % U;
+                const int blk = W13 ? local % run.nb : local / U;
                 GItem gi;
-                gi.k = k;
+                gi.k = run.first + blk;
                 gi.u = u;
-                gi.ci = ci;
+                gi.nstream = W13 ? 2 : w2_pair_width(u, nrb);
+                gi.pair_base = run.off + blk * kGN;
+                gi.nv = min(kGN, run.cnt - blk * kGN);
+                gi.n = (gi.nv + 15) & ~15;
                 sh->items[nitem % kGItemRing] = gi;
+                mbar_arrive(&sh->itembar[nitem % kGItemRing]);
                 ++nitem;
-                const int narrow = ci.nv <= kGNarrow;
-                const int STB = supertile_bytes(bits, group);
-                const int pw = W13 ? 2 : w2_pair_width(u, nrb);
-                const uint8_t *wsrc = p.packed + p.mat_off[e][W13 ? 0 : 2] +
+                const int STB = supertile_bytes(run.bits, group);
+                const uint8_t *wsrc = p.packed + p.mat_off[run.e][W13 ? 0 : 2] +
                                       supertile_off(W13 ? 0 : 2, W13 ? u : 2 * u, 0, KTm, nrb, STB);
-                const uint8_t *isrc = img_base + (size_t)k * KTm * kImgBytes;
+                const uint32_t wb = (uint32_t)(gi.nstream * STB);
+                int next = total;
                 for (int kt = 0; kt < KTm; ++kt, ++it) {
-                    const int slot = it % kGSlots;
-                    if (it >= kGSlots && !g_wait(&sh->empty[slot], ((it / kGSlots) - 1) & 1, p, sh)) {
+                    if (it >= geo.nw && !g_wait(&sh->wempty[slot], phase ^ 1u, p, sh)) {
                         ok = false;
                         break;
                     }
-                    GStage &st = sh->stage[slot];
-                    st.item = item;
-                    st.kt = kt;
-                    st.first = kt == 0;
-                    st.last = kt == KTm - 1;
-                    st.k = k;
-                    st.u = u;
-                    st.narrow = narrow;
-                    st.ci = ci;
-                    uint8_t *dst = ring + (size_t)slot * kGStage;
-                    const uint8_t *src = isrc + (size_t)kt * kImgBytes;
-                    const uint32_t wb = (uint32_t)(pw * STB);
-                    if (narrow) {
-                        // rows 0..63 of both 64-column atoms: the first 8 KB of each 16 KB
-                        mbar_arrive_expect_tx(&sh->full[slot], (uint32_t)(kImgBytes / 2) + wb);
-                        bulk_g2s(dst, src, kImgBytes / 4, &sh->full[slot]);
-                        bulk_g2s(dst + kImgBytes / 2, src + kImgBytes / 2, kImgBytes / 4, &sh->full[slot]);
-                    } else {
-                        mbar_arrive_expect_tx(&sh->full[slot], (uint32_t)kImgBytes + wb);
-                        bulk_g2s(dst, src, kImgBytes, &sh->full[slot]);
-                    }
+                    sh->wst[slot] = GWStage{item, run.bits, gi.nstream,
+                                            gi.n | (kt == 0 ? kInfoFirst : 0) | (kt == KTm - 1 ? kInfoLast : 0) |
+                                                (gi.nstream == 1 ? kInfoLone : 0)};
+                    uint8_t *dst = smem + geo.w0 + slot * geo.wslot;
+                    mbar_arrive_expect_tx(&sh->wfull[slot], wb);
                     // W1,W3 weights are read by the CTAs of one row block at about
                     // the same time: evict-first; a W2 row-block pair's weights come
                     // back for every token block of the expert: normal policy
-                    if (W13) bulk_g2s_stream(dst + kImgBytes, wsrc + (size_t)kt * pw * STB, wb, &sh->full[slot], pol);
-                    else bulk_g2s(dst + kImgBytes, wsrc + (size_t)kt * pw * STB, wb, &sh->full[slot]);
-                    sh->issued = it + 1;
+                    if (W13) bulk_g2s_stream(dst, wsrc + (size_t)kt * wb, wb, &sh->wfull[slot], pol);
+                    else bulk_g2s(dst, wsrc + (size_t)kt * wb, wb, &sh->wfull[slot]);
+                    sh->wissued = it + 1;
+                    // the next item's claim overlaps this item's last copies
+                    if (kt == max(0, KTm - 2)) next = atomicAdd(counter, 1);
+                    if (++slot == geo.nw) {
+                        slot = 0;
+                        phase ^= 1u;
+                    }
+                }
+                item = next;
+            }
+            if (ok) {
+                pdl_trigger();  // the CTA takes no further item: the next kernel may launch
+                sh->items[nitem % kGItemRing].k = -1;
+                mbar_arrive(&sh->itembar[nitem % kGItemRing]);
+                // two end markers: each parity's converters take every other step
+                for (int m = 0; m < 2; ++m, ++it) {
+                    if (it >= geo.nw && !g_wait(&sh->wempty[slot], phase ^ 1u, p, sh)) break;
+                    sh->wst[slot].item = -1;
+                    mbar_arrive(&sh->wfull[slot]);
+                    if (++slot == geo.nw) {
+                        slot = 0;
+                        phase ^= 1u;
+                    }
                 }
             }
-            // two end markers, one for each converter group (each takes every
-            // other stage)
-            for (int m = 0; ok && m < 2; ++m, ++it) {
-                const int slot = it % kGSlots;
-                if (it >= kGSlots && !g_wait(&sh->empty[slot], ((it / kGSlots) - 1) & 1, p, sh)) break;
-                sh->stage[slot].item = -1;
-                mbar_arrive(&sh->full[slot]);
+        }
+    } else if (warp == kGImgProd) {
+        // ------------------------------------------------------ image producer --
+        if (lane == 0) {
+            int it = 0, slot = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int n = 0; ok; ++n) {
+                if (!g_wait(&sh->itembar[n % kGItemRing], (n / kGItemRing) & 1, p, sh)) break;
+                const GItem gi = sh->items[n % kGItemRing];
+                if (gi.k < 0) break;
+                const uint8_t *src = img_base + (size_t)gi.k * KTm * kImgBytes;
+                const uint32_t ab = (uint32_t)gi.n * 128u;  // rows 0 .. n - 1 of an atom
+                for (int kt = 0; kt < KTm; ++kt, ++it, src += kImgBytes) {
+                    if (it >= geo.ni && !g_wait(&sh->iempty[slot], phase ^ 1u, p, sh)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t *dst = smem + geo.img0 + slot * 2 * geo.atom;
+                    mbar_arrive_expect_tx(&sh->ifull[slot], 2 * ab);
+                    if (gi.n == kGN) {
+                        bulk_g2s(dst, src, 2 * ab, &sh->ifull[slot]);
+                    } else {
+                        bulk_g2s(dst, src, ab, &sh->ifull[slot]);
+                        bulk_g2s(dst + geo.atom, src + kImgBytes / 2, ab, &sh->ifull[slot]);
+                    }
+                    sh->iissued = it + 1;
+                    if (++slot == geo.ni) {
+                        slot = 0;
+                        phase ^= 1u;
+                    }
+                }
             }
         }
-    } else if (warp < kGEpi0 || (warp >= 8 && warp < 12)) {
+    } else if (warp < kGConv) {
         // ---------------------------------------------------------- converters --
-        // group cg takes stages cg, cg + 2, ... into A buffer cg; warp q of the
-        // group owns tensor-memory lanes 32q .. 32q + 31 (tiles 2q, 2q + 1)
-        const int q = warp & 3, cg = warp >> 3;
-        const uint32_t abuf = tbase + 256u + 128u * (uint32_t)cg;
-        for (int it = cg, n = 0;; it += 2, ++n) {
-            const int slot = it % kGSlots;
-            if (!g_wait(&sh->full[slot], (it / kGSlots) & 1, p, sh)) break;
-            const GStage st = sh->stage[slot];
-            if (st.item < 0) {
-                // the MMA warps wait on afull only: pass the end marker on, once
-                // the MMAs of the group's previous stage are done (so that afull
-                // never completes a phase before the MMA warps waited for the one
-                // before it)
-                if (n > 0 && !g_wait(&sh->aempty[cg], (uint32_t)((n - 1) & 1), p, sh)) break;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh->afull[cg]);
-                break;
+        // warp q of the group (stream cg, parity b) converts tiles 2q, 2q + 1 of the
+        // stream (tensor-memory lanes 32q .. 32q + 31) in every other step, into the
+        // stream's A buffer b
+        const int q = warp & 3, cg = (warp >> 2) & 1, b = warp >> 3;
+        const uint32_t abuf = tbase + 256u + 128u * (uint32_t)cg + 64u * (uint32_t)b + ((uint32_t)(32 * q) << 16);
+        int slot = b;
+        uint32_t phase = 0;
+        for (int n = 0;; ++n) {
+            if (!g_wait(&sh->wfull[slot], phase, p, sh)) break;
+            const GWStage st = sh->wst[slot];
+            const bool active = st.item >= 0 && cg < st.nstream;
+            RawTile<GPT> ta, tb;
+            if (active) {
+                const int TB = tile_bytes(st.bits, group);
+                const uint8_t *w = smem + geo.w0 + slot * geo.wslot + cg * (kTilesPerBlock * TB) + 2 * q * TB;
+                load_raw<GPT>(w, st.bits, lane, ta);
+                load_raw<GPT>(w + TB, st.bits, lane, tb);
             }
-            const int bits = st.ci.bits, STB = supertile_bytes(bits, group), TB = tile_bytes(bits, group);
-            const int nstream = W13 ? 2 : w2_pair_width(st.u, nrb);
-            const uint8_t *w = ring + (size_t)slot * kGStage + kImgBytes;
-            if (!convert_stage<GPT>(w, bits, nstream, STB, TB, q, lane, abuf, n > 0, &sh->aempty[cg],
-                                    (uint32_t)((n - 1) & 1), p, sh))
-                break;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh->wempty[slot]);  // the packed words are in registers
+            slot += 2;
+            if (slot >= geo.nw) {
+                slot -= geo.nw;
+                phase ^= 1u;
+            }
+            uint32_t v[32];
+            if (active) convert_regs<GPT>(ta, st.bits, v);
+            // the MMAs that read this buffer last are done (and afull's phase of that
+            // step has been waited for)
+            if (n > 0 && !g_wait(&sh->aempty[cg][b], (uint32_t)((n - 1) & 1), p, sh)) break;
+            if (active) {
+                tc_fence_after();
+                tmem_st_16x256_x8(abuf, v);
+                convert_regs<GPT>(tb, st.bits, v);
+                tmem_st_16x256_x8(abuf + (16u << 16), v);
+                tmem_st_wait();
+            }
+            if (q == 0 && lane == 0) sh->ainfo[cg][b] = st.item < 0 ? kInfoEnd : st.info;
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&sh->afull[cg]);
-                mbar_arrive(&sh->empty[slot]);
-            }
+            if (lane == 0) mbar_arrive(&sh->afull[cg][b]);
+            if (st.item < 0) break;
         }
     } else if (warp >= kGMma && warp < kGMma + kGMmaN) {
         // ----------------------------------------------------------------- MMA --
+        // The whole warp runs the loop, one elected lane issues (elect_one).
         const int mx = warp - kGMma;  // the weight stream this warp multiplies
-        if (lane == 0) {
-            int nitem = 0;
-            for (int it = 0;; ++it) {
-                const int slot = it % kGSlots, b = it & 1;
-                // the stage's converter group arrives after it saw the copies land
-                if (!g_wait(&sh->afull[b], (it >> 1) & 1, p, sh)) break;
-                const GStage st = sh->stage[slot];
-                if (st.item < 0) break;
-                if (st.first && nitem > 0 && !g_wait(&sh->dempty, (nitem - 1) & 1, p, sh)) break;
-                tc_fence_after();
-                const int nstream = W13 ? 2 : w2_pair_width(st.u, nrb);
-                if (mx < nstream) {
-                    const uint32_t idesc = umma_idesc_f16(128, st.narrow ? kGNarrow : kGN);
-                    const uint8_t *img = ring + (size_t)slot * kGStage;
-                    const uint32_t abuf = tbase + 256u + 128u * (uint32_t)b + 64u * (uint32_t)mx;
+        int nitem = 0, slot = 0;
+        uint32_t phase = 0;
+        for (int it = 0;; ++it) {
+            const int b = it & 1;
+            if (!warp_wait(&sh->afull[mx][b], (it >> 1) & 1, p, sh)) break;
+            const int info = sh->ainfo[mx][b];
+            if (info & kInfoEnd) break;
+            const int par = nitem % nbuf, use = nitem / nbuf;
+            if ((info & kInfoFirst) && use > 0 && !warp_wait(&sh->dempty[par], (use - 1) & 1, p, sh)) break;
+            if (!warp_wait(&sh->ifull[slot], phase, p, sh)) break;
+            tc_fence_after();
+            const uint32_t idesc = umma_idesc_f16(128, info & kInfoN);
+            const uint64_t bd = umma_desc_sw128(smem + geo.img0 + slot * 2 * geo.atom);
+            const uint64_t bd1 = bd + (uint64_t)(geo.atom >> 4);
+            const uint32_t abuf = tbase + 256u + 128u * (uint32_t)mx + 64u * (uint32_t)b;
+            const uint32_t d = tbase + 128u * (uint32_t)mx + (uint32_t)(kGNarrow * par);
+            if (elect_one()) {
+                // (a lone W2 block's second stream multiplies nothing: its converters
+                // stored no tile and its accumulator is not read)
+                if (mx == 0 || !(info & kInfoLone)) {
 #pragma unroll
-                    for (int s = 0; s < 8; ++s) {
-                        const uint64_t bd = umma_desc_sw128(img + (s >> 2) * 16384 + (s & 3) * 32);
-                        umma_f16_ts(tbase + 128u * (uint32_t)mx, abuf + 8u * (uint32_t)s, bd, idesc,
-                                    !(st.first && s == 0));
-                    }
+                    for (int s = 0; s < 8; ++s)
+                        umma_f16_ts(d, abuf + 8u * (uint32_t)s, (s < 4 ? bd : bd1) + (uint64_t)(2 * (s & 3)), idesc,
+                                    s > 0 || !(info & kInfoFirst));
                 }
-                umma_commit(&sh->aempty[b]);
-                umma_commit(&sh->empty[slot]);
-                if (st.last) {
-                    umma_commit(&sh->dfull);
-                    ++nitem;
-                }
+                umma_commit(&sh->aempty[mx][b]);
+                umma_commit(&sh->iempty[slot]);
+                if (info & kInfoLast) umma_commit(&sh->dfull[par]);
             }
-            // every MMA of both warps has completed (and with it every commit to
-            // dfull) before the epilogue is told that no item follows and before
-            // TMEM is released
-            umma_commit(&sh->drain);
-            const uint64_t t0 = globaltimer_ns();
-            while (!mbar_try_wait(&sh->drain, 0))
-                if (globaltimer_ns() - t0 > p.timeout_ns) break;
-            // the epilogue has taken the last item before dfull completes once more,
-            // so that it never sees two completions of dfull in one wait
-            if (nitem == 0 || g_wait(&sh->dempty, (nitem - 1) & 1, p, sh)) {
-                if (mx == 0) sh->end_items = nitem;
-                mbar_arrive(&sh->dfull);
+            __syncwarp();
+            if (info & kInfoLast) ++nitem;
+            if (++slot == geo.ni) {
+                slot = 0;
+                phase ^= 1u;
             }
         }
-    } else if (warp >= kGEpi0 && warp < kGEpi0 + 4) {
+        // every MMA of both warps has completed (and with it every commit to
+        // dfull) before the epilogue is told that no item follows and before
+        // TMEM is released
+        __syncwarp();
+        if (elect_one()) umma_commit(&sh->drain);
+        __syncwarp();
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(&sh->drain, 0))
+            if (globaltimer_ns() - t0 > p.timeout_ns) break;
+        __syncwarp();
+        // the epilogue has taken the last item of this accumulator set before its
+        // dfull completes once more, so that it never sees two completions of one
+        // barrier in one wait
+        const int par = nitem % nbuf, use = nitem / nbuf;
+        if ((use == 0 || warp_wait(&sh->dempty[par], (use - 1) & 1, p, sh)) && lane == 0) {
+            if (mx == 0) sh->end_items = nitem;
+            mbar_arrive(&sh->dfull[par]);
+        }
+    } else {
         // ------------------------------------------------------------ epilogue --
         const int ew = warp - kGEpi0;   // tensor-memory lanes 32 ew .. 32 ew + 31
         const int row = 32 * ew + lane;  // row of the 128-row block
         const int tid = threadIdx.x - 32 * kGEpi0;
         int uses = 0;
         for (int ic = 0;; ++ic) {
-            if (!g_wait(&sh->dfull, ic & 1, p, sh)) break;
+            const int par = ic % nbuf;
+            if (!g_wait(&sh->dfull[par], (ic / nbuf) & 1, p, sh)) break;
             if (ic >= sh->end_items) break;
             tc_fence_after();
             const GItem gi = sh->items[ic % kGItemRing];
-            const uint32_t lane_addr = (uint32_t)(32 * ew) << 16;
+            const uint32_t dbase = tbase + ((uint32_t)(32 * ew) << 16) + (uint32_t)(kGNarrow * par);
             if (W13) {
-                // h of the thread's row for all 128 pairs, packed, so that D is released
-                // before the image is written
-                uint32_t hp[kGN / 2];
+                // h of the thread's row, 64 pairs at a time packed in registers, so that D
+                // is released before the last of the image is written (rows nv .. n - 1
+                // of the block's x image are zero, so their h is)
                 bool bad = false;
+#pragma unroll 1
+                for (int h0 = 0; h0 < gi.n; h0 += 64) {
+                    uint32_t hp[32];
 #pragma unroll
-                for (int n0 = 0; n0 < kGN; n0 += 16) {
-                    if (n0 >= gi.ci.nv) {  // no pair of the block in these columns: zero rows
+                    for (int n0 = 0; n0 < 64; n0 += 16) {
+                        if (h0 + n0 >= gi.n) continue;
+                        uint32_t g[16], v[16];
+                        tmem_ld_x16_nowait(dbase + (uint32_t)(h0 + n0), g);
+                        tmem_ld_x16_nowait(dbase + 128u + (uint32_t)(h0 + n0), v);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int i = 0; i < 16; i += 2) hp[(n0 + i) / 2] = 0u;
-                        continue;
+                        for (int i = 0; i < 16; i += 2) {
+                            const float v0 = silu(__uint_as_float(g[i])) * __uint_as_float(v[i]);
+                            const float v1 = silu(__uint_as_float(g[i + 1])) * __uint_as_float(v[i + 1]);
+                            bad |= !(fabsf(v0) <= 65504.f) || !(fabsf(v1) <= 65504.f);
+                            hp[(n0 + i) / 2] = h2_bits(__floats2half2_rn(v0, v1));
+                        }
                     }
-                    uint32_t g[16], v[16];
-                    tmem_ld_x16_nowait(tbase + lane_addr + (uint32_t)n0, g);
-                    tmem_ld_x16_nowait(tbase + lane_addr + 128u + (uint32_t)n0, v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (h0 + 64 >= gi.n) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sh->dempty[par]);
+                    }
 #pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        const float h0 = silu(__uint_as_float(g[i])) * __uint_as_float(v[i]);
-                        const float h1 = silu(__uint_as_float(g[i + 1])) * __uint_as_float(v[i + 1]);
-                        bad |= !(fabsf(h0) <= 65504.f) || !(fabsf(h1) <= 65504.f);
-                        hp[(n0 + i) / 2] = h2_bits(__floats2half2_rn(h0, h1));
+                    for (int n0 = 0; n0 < 64; n0 += 16) {
+                        if (h0 + n0 >= gi.n) continue;
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2) {
+                            const __half2 h = bits_h2(hp[(n0 + i) / 2]);
+                            *reinterpret_cast<__half *>(staging + img_off(h0 + n0 + i, row, geo.atom)) = __low2half(h);
+                            *reinterpret_cast<__half *>(staging + img_off(h0 + n0 + i + 1, row, geo.atom)) = __high2half(h);
+                        }
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh->dempty);
                 if (bad) set_status(p.status, MC_ERR_RANGE);
-#pragma unroll
-                for (int i = 0; i < kGN / 2; ++i) {
-                    const __half2 h = bits_h2(hp[i]);
-                    *reinterpret_cast<__half *>(staging + img_off(2 * i, row)) = __low2half(h);
-                    *reinterpret_cast<__half *>(staging + img_off(2 * i + 1, row)) = __high2half(h);
-                }
                 // the image of W2's column step gi.u for token block gi.k
                 if (!epi_sync(p, sh, lane, uses)) break;
-                uint4 *dst = reinterpret_cast<uint4 *>(p.himg + ((size_t)gi.k * (p.F / kTileK) + gi.u) * kImgBytes);
-                const uint4 *src = reinterpret_cast<const uint4 *>(staging);
-                for (int i = tid; i < kImgBytes / 16; i += 128) dst[i] = src[i];
+                uint8_t *dst = p.himg + ((size_t)gi.k * (p.F / kTileK) + gi.u) * kImgBytes;
+                for (int i = tid; i < gi.n * 8; i += 128) {
+                    reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(staging)[i];
+                    reinterpret_cast<uint4 *>(dst + kImgBytes / 2)[i] =
+                        reinterpret_cast<const uint4 *>(staging + geo.atom)[i];
+                }
                 if (!epi_sync(p, sh, lane, uses)) break;
             } else {
-                const int nstream = w2_pair_width(gi.u, nrb);
                 float *out = p.opart;
-                for (int x = 0; x < nstream; ++x) {
+                for (int x = 0; x < gi.nstream; ++x) {
                     const int blk = 2 * gi.u + x;
-                    for (int n0 = 0; n0 < gi.ci.nv; n0 += 16) {
+                    for (int n0 = 0; n0 < gi.nv; n0 += 16) {
                         float v[16];
-                        tmem_ld_x16(tbase + lane_addr + 128u * (uint32_t)x + (uint32_t)n0, v);
+                        tmem_ld_x16(dbase + 128u * (uint32_t)x + (uint32_t)n0, v);
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
-                            if (n0 + i < gi.ci.nv)
-                                out[(size_t)(gi.ci.pair_base + n0 + i) * p.H + blk * kBlockRows + row] = v[i];
+                            if (n0 + i < gi.nv)
+                                out[(size_t)(gi.pair_base + n0 + i) * p.H + blk * kBlockRows + row] = v[i];
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&sh->dempty);
+                if (lane == 0) mbar_arrive(&sh->dempty[par]);
             }
         }
     }
 
     tc_fence_before();
     __syncthreads();
+    // On an abort, let copies that were issued but never consumed land before the
+    // CTA's shared memory is released (bounded).
     if (threadIdx.x == 0 && sh->abort) {
-        for (int it = max(0, sh->issued - kGSlots); it < sh->issued; ++it) {
+        for (int it = max(0, sh->wissued - geo.nw); it < sh->wissued; ++it) {
             const uint64_t t0 = globaltimer_ns();
-            while (!mbar_try_wait(&sh->full[it % kGSlots], (it / kGSlots) & 1))
+            while (!mbar_try_wait(&sh->wfull[it % geo.nw], (it / geo.nw) & 1))
+                if (globaltimer_ns() - t0 > p.timeout_ns) break;
+        }
+        for (int it = max(0, sh->iissued - geo.ni); it < sh->iissued; ++it) {
+            const uint64_t t0 = globaltimer_ns();
+            while (!mbar_try_wait(&sh->ifull[it % geo.ni], (it / geo.ni) & 1))
                 if (globaltimer_ns() - t0 > p.timeout_ns) break;
         }
     }

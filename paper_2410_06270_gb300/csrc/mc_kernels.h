@@ -78,6 +78,7 @@ struct ExpertParams {
     int E, H, F, group;
     const ChunkInfo *chunks;
     const int32_t *nchunks;
+    const int32_t *offsets;  // [E+1] pairs before each expert (prefill path)
     int32_t *counters;
     const __nv_bfloat16 *x;  // [T, H]
     const int32_t *perm;     // [P]

@@ -95,6 +95,18 @@ __device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 
+// True in one lane of the (converged) warp, the same one every time.  MMAs issued
+// under `if (elect_one())` in warp-uniform code take their operands from uniform
+// registers; under `if (lane == 0)` every operand is moved there first, instruction
+// by instruction: 8 issues took 541 cycles alone and 859 beside 16 busy warps, with
+// the elected lane and descriptors formed by adding constants 160 and 249.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0;
+}
+
 // Arrive once on `bar` when every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
