@@ -170,6 +170,9 @@ __device__ __forceinline__ bool g_header_ok(const ExpertParams &p)
     return ok;
 }
 
+__device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t *>(&v); }
+__device__ __forceinline__ __half2 bits_h2(uint32_t v) { return *reinterpret_cast<const __half2 *>(&v); }
+
 // ------------------------------------------------------------------ x image --
 __global__ void __launch_bounds__(256) x_img_kernel(ExpertParams p)
 {
@@ -224,8 +227,6 @@ __device__ __forceinline__ uint32_t pair_offset_bits(int j)
     return MC_C(25 - f);
 }
 
-__device__ __forceinline__ uint32_t h2_bits(__half2 v) { return *reinterpret_cast<const uint32_t *>(&v); }
-__device__ __forceinline__ __half2 bits_h2(uint32_t v) { return *reinterpret_cast<const __half2 *>(&v); }
 
 // The code words and (scale, zero) pairs of one lane's part of a tile, as stored.
 template <int GPT>
@@ -269,9 +270,9 @@ __device__ __forceinline__ void convert_tile(const RawTile<GPT> &t, uint32_t (&o
 #pragma unroll
     for (int qd = 0; qd < 4; ++qd) {
         uint32_t r[8];
-        if (BITS == 1) cvt1_half(t.w[4 + (qd >> 1)], 8 * (qd & 1), r);
-        if (BITS == 2) cvt2(t.w[qd], r);
-        if (BITS == 3) cvt3(t.w, qd, r);
+        if constexpr (BITS == 1) cvt1_half(t.w[4 + (qd >> 1)], 8 * (qd & 1), r);
+        if constexpr (BITS == 2) cvt2(t.w[qd], r);
+        if constexpr (BITS == 3) cvt3(t.w, qd, r);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int j = 8 * qd + i, s = j >> 2, rho = j & 3;
@@ -297,12 +298,23 @@ __device__ __forceinline__ void tmem_st_16x256_x8(uint32_t taddr, const uint32_t
         : "memory");
 }
 
-template <int GPT>
-__device__ __forceinline__ void convert_regs(const RawTile<GPT> &t, int bits, uint32_t (&v)[32])
+// A step's two tiles of one converter warp: converted and stored, the first store
+// after the MMAs have read the buffer.  One code path per width from the packed words
+// to the store: tcgen05.st takes 32 consecutive registers, and a store shared by the
+// widths' branches costs a move per register.  False once the CTA aborted.
+template <int BITS, int GPT>
+__device__ __forceinline__ bool convert_store(const RawTile<GPT> &ta, const RawTile<GPT> &tb, uint32_t abuf, bool wait,
+                                              uint64_t *aempty, uint32_t parity, const ExpertParams &p, GShared *sh)
 {
-    if (bits == 1) convert_tile<1, GPT>(t, v);
-    else if (bits == 2) convert_tile<2, GPT>(t, v);
-    else convert_tile<3, GPT>(t, v);
+    uint32_t v[32];
+    convert_tile<BITS, GPT>(ta, v);
+    if (wait && !g_wait(aempty, parity, p, sh)) return false;
+    tc_fence_after();
+    tmem_st_16x256_x8(abuf, v);
+    convert_tile<BITS, GPT>(tb, v);
+    tmem_st_16x256_x8(abuf + (16u << 16), v);
+    tmem_st_wait();
+    return true;
 }
 
 // ------------------------------------------------------------- epilogue --
@@ -565,18 +577,17 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_kernel(ExpertParams p)
                 slot -= geo.nw;
                 phase ^= 1u;
             }
-            uint32_t v[32];
-            if (active) convert_regs<GPT>(ta, st.bits, v);
             // the MMAs that read this buffer last are done (and afull's phase of that
             // step has been waited for)
-            if (n > 0 && !g_wait(&sh->aempty[cg][b], (uint32_t)((n - 1) & 1), p, sh)) break;
-            if (active) {
-                tc_fence_after();
-                tmem_st_16x256_x8(abuf, v);
-                convert_regs<GPT>(tb, st.bits, v);
-                tmem_st_16x256_x8(abuf + (16u << 16), v);
-                tmem_st_wait();
-            }
+            const bool wait = n > 0;
+            const uint32_t par = (uint32_t)((n - 1) & 1);
+            uint64_t *ae = &sh->aempty[cg][b];
+            bool ok;
+            if (!active) ok = !wait || g_wait(ae, par, p, sh);
+            else if (st.bits == 1) ok = convert_store<1, GPT>(ta, tb, abuf, wait, ae, par, p, sh);
+            else if (st.bits == 2) ok = convert_store<2, GPT>(ta, tb, abuf, wait, ae, par, p, sh);
+            else ok = convert_store<3, GPT>(ta, tb, abuf, wait, ae, par, p, sh);
+            if (!ok) break;
             if (q == 0 && lane == 0) sh->ainfo[cg][b] = st.item < 0 ? kInfoEnd : st.info;
             tc_fence_before();
             __syncwarp();
