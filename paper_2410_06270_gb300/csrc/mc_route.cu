@@ -8,6 +8,7 @@
 //   rows, 16 bytes each) before it uses any, so a round costs one memory round
 //   trip; the partial logits meet in shared memory, warp 0 adds them up and
 //   thread 0 takes the decision in fp32.
+// route_multi_kernel (from 153 tokens): four tokens per CTA, the gate loaded once.
 // route_cluster_kernel (T <= 16): the same as one thread-block cluster, the
 //   decisions gathered in CTA 0's shared memory and placed by its first warp.
 // permute_kernel: one CTA; histogram, exclusive scan and a stable placement with
@@ -58,6 +59,62 @@ __device__ __forceinline__ float route_row_inv(const RouteParams &p, int t, uint
 #pragma unroll
     for (int w = 0; w < 8; ++w) tot += red[w];
     return rsqrtf(tot / p.H + p.eps);
+}
+
+// One thread: token t's decision from its logits l (fp32) and its mask byte, written to
+// the outputs (and to `sink`, if given: e0, e1, pruned at 3 t).
+__device__ __forceinline__ void route_decide(const RouteParams &p, int t, const float (&l)[kMaxE], int mask, int *sink)
+{
+    const int E = p.E;
+    // top-2 on fp32 logits, lower index wins ties
+    int e0 = 0;
+    float b0 = l[0];
+#pragma unroll
+    for (int e = 1; e < kMaxE; ++e)
+        if (e < E && l[e] > b0) {
+            b0 = l[e];
+            e0 = e;
+        }
+    int e1 = -1;
+    float b1 = 0.f;
+#pragma unroll
+    for (int e = 0; e < kMaxE; ++e)
+        if (e < E && e != e0 && (e1 < 0 || l[e] > b1)) {
+            b1 = l[e];
+            e1 = e;
+        }
+    const float d = b0 - b1;  // >= 0
+    const float r = __expf(-d);     // = p1 / p0
+    float w0 = 1.f / (1.f + r), w1 = r / (1.f + r);
+    const bool drop = mask == 2, prot = mask != 0 && !drop;
+    int prune = !prot && (d > p.neg_log_mu);
+    if (prune) {
+        w0 = 1.f;
+        w1 = 0.f;
+    }
+    if (drop) {  // no expert: weights (0, 0), pruned = 2
+        w0 = w1 = 0.f;
+        prune = 2;
+    }
+    if (sink) {
+        sink[3 * t] = e0;
+        sink[3 * t + 1] = e1;
+        sink[3 * t + 2] = prune;
+    }
+    p.idx[2 * t] = e0;
+    p.idx[2 * t + 1] = e1;
+    p.w[2 * t] = w0;
+    p.w[2 * t + 1] = w1;
+    p.pruned[t] = (uint8_t)prune;
+    if (p.idx_out) {
+        p.idx_out[2 * t] = e0;
+        p.idx_out[2 * t + 1] = e1;
+    }
+    if (p.w_out) {
+        p.w_out[2 * t] = w0;
+        p.w_out[2 * t + 1] = w1;
+    }
+    if (p.pruned_out) p.pruned_out[t] = (uint8_t)prune;
 }
 
 // The logits of token t by the whole CTA; thread 0 takes the decision and writes
@@ -151,55 +208,7 @@ __device__ __forceinline__ void route_token(const RouteParams &p, int t, int *si
 #pragma unroll
     for (int e = 0; e < kMaxE; ++e) l[e] = __shfl_sync(0xffffffffu, le, e);
     if (lane != 0) return;
-    // top-2 on fp32 logits, lower index wins ties
-    int e0 = 0;
-    float b0 = l[0];
-#pragma unroll
-    for (int e = 1; e < kMaxE; ++e)
-        if (e < E && l[e] > b0) {
-            b0 = l[e];
-            e0 = e;
-        }
-    int e1 = -1;
-    float b1 = 0.f;
-#pragma unroll
-    for (int e = 0; e < kMaxE; ++e)
-        if (e < E && e != e0 && (e1 < 0 || l[e] > b1)) {
-            b1 = l[e];
-            e1 = e;
-        }
-    const float d = b0 - b1;  // >= 0
-    const float r = __expf(-d);     // = p1 / p0
-    float w0 = 1.f / (1.f + r), w1 = r / (1.f + r);
-    const bool drop = mask == 2, prot = mask != 0 && !drop;
-    int prune = !prot && (d > p.neg_log_mu);
-    if (prune) {
-        w0 = 1.f;
-        w1 = 0.f;
-    }
-    if (drop) {  // no expert: weights (0, 0), pruned = 2
-        w0 = w1 = 0.f;
-        prune = 2;
-    }
-    if (sink) {
-        sink[3 * t] = e0;
-        sink[3 * t + 1] = e1;
-        sink[3 * t + 2] = prune;
-    }
-    p.idx[2 * t] = e0;
-    p.idx[2 * t + 1] = e1;
-    p.w[2 * t] = w0;
-    p.w[2 * t + 1] = w1;
-    p.pruned[t] = (uint8_t)prune;
-    if (p.idx_out) {
-        p.idx_out[2 * t] = e0;
-        p.idx_out[2 * t + 1] = e1;
-    }
-    if (p.w_out) {
-        p.w_out[2 * t] = w0;
-        p.w_out[2 * t + 1] = w1;
-    }
-    if (p.pruned_out) p.pruned_out[t] = (uint8_t)prune;
+    route_decide(p, t, l, mask, sink);
 }
 
 template <bool NORM>
@@ -208,6 +217,122 @@ __global__ void __launch_bounds__(kRouteThreads) route_kernel(RouteParams p)
     pdl_trigger();
     pdl_wait();
     route_token<NORM>(p, blockIdx.x);
+}
+
+// kRouteTT tokens per CTA, for calls with many tokens and at most 8 experts: the gate
+// rows are loaded once for all of them (64 KB of L2 reads per CTA at H = 4096, which
+// one CTA per token repeated 4096 times), and a warp's 8 partial logits of a token are
+// summed over the lanes by halving exchanges (9 shuffles instead of 40), every sum over
+// the same operands as in route_token, so the logits are bit for bit the same.
+// route_kernel's 128 registers leave room for one CTA per SM, so from 153 tokens on it
+// takes a second wave: 256 tokens 12.1 -> 8.6 us between events (an empty launch reads
+// ~5), 1019 tokens 26.7 -> 12.6 us, 4096 tokens 87 -> 29 us.
+constexpr int kRouteTT = 4, kRouteTTMinT = 153, kRouteTTMaxE = 8;
+
+__global__ void __launch_bounds__(kRouteThreads) route_multi_kernel(RouteParams p)
+{
+    __shared__ float part[kRouteThreads / 32][kRouteTT][kRouteTTMaxE];
+    pdl_trigger();
+    pdl_wait();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int H = p.H, E = p.E, t0 = blockIdx.x * kRouteTT;
+    const int t = t0 + warp;  // the token that this warp (of the first kRouteTT) decides
+    const int mask = warp < kRouteTT && t < p.T && lane == 0 && p.protect != nullptr ? p.protect[t] : 0;
+    float acc[kRouteTT][kRouteTTMaxE];
+#pragma unroll
+    for (int k = 0; k < kRouteTT; ++k)
+#pragma unroll
+        for (int e = 0; e < kRouteTTMaxE; ++e) acc[k][e] = 0.f;
+    for (int c0 = 8 * threadIdx.x; c0 < H; c0 += 8 * kRouteThreads) {
+        uint4 raw[kRouteTT], gr[kRouteTTMaxE];
+#pragma unroll
+        for (int k = 0; k < kRouteTT; ++k)  // (past the last token: the last one again, unused)
+            raw[k] = *reinterpret_cast<const uint4 *>(p.x + (size_t)min(t0 + k, p.T - 1) * H + c0);
+#pragma unroll
+        for (int e = 0; e < kRouteTTMaxE; ++e)
+            gr[e] = e < E ? *reinterpret_cast<const uint4 *>(p.gate + (size_t)e * H + c0) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int k = 0; k < kRouteTT; ++k) {
+            const __nv_bfloat162 *x2 = reinterpret_cast<const __nv_bfloat162 *>(&raw[k]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 xf = __bfloat1622float2(x2[i]);
+#pragma unroll
+                for (int e = 0; e < kRouteTTMaxE; ++e) {
+                    const float2 gf = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162 *>(&gr[e])[i]);
+                    acc[k][e] = fmaf(xf.x, gf.x, acc[k][e]);
+                    acc[k][e] = fmaf(xf.y, gf.y, acc[k][e]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kRouteTT; ++k) {
+        // lanes m apart add the same two partials either way, so each keeps half of the
+        // experts: after 16, 8 and 4 lane l holds expert l / 4
+        float v4[4], v2[2], v;
+        const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float give = h16 ? acc[k][i] : acc[k][4 + i], keep = h16 ? acc[k][4 + i] : acc[k][i];
+            v4[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float give = h8 ? v4[i] : v4[2 + i], keep = h8 ? v4[2 + i] : v4[i];
+            v2[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+        }
+        v = (h4 ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, h4 ? v2[0] : v2[1], 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        if ((lane & 3) == 0) part[warp][k][lane >> 2] = v;
+    }
+    __syncthreads();
+    if (warp >= kRouteTT || t >= p.T) return;
+    float le = 0.f;
+    if (lane < E)
+        for (int w = 0; w < kRouteThreads / 32; ++w) le += part[w][warp][lane];
+    float l[kMaxE];
+#pragma unroll
+    for (int e = 0; e < kMaxE; ++e) l[e] = __shfl_sync(0xffffffffu, le, e);
+    if (lane == 0) route_decide(p, t, l, mask, nullptr);
+}
+
+// Thread e < E: expert e's offset (also in run[e]) and work chunks from the counts; the
+// chunk total and the work counters.
+__device__ __forceinline__ void permute_lists(const PermuteParams &p, const int *cnt, int *run, const int *nbits)
+{
+    const int tid = threadIdx.x;
+    if (tid < p.E) {
+        // expert tid: its offset, and the index of its first work chunk in the
+        // order the expert kernels take them (more bits first, then by expert)
+        const int e = tid, be = nbits[e], ce = cnt[e];
+        int off = 0, k0 = 0;
+        for (int f = 0; f < p.E; ++f) {
+            const int cf = cnt[f], bf = nbits[f];
+            if (f < e) off += cf;
+            if (bf > be || (bf == be && f < e)) k0 += (cf + p.chunk - 1) / p.chunk;
+        }
+        p.offsets[e] = off;
+        run[e] = off;
+        if (e == p.E - 1) p.offsets[p.E] = off + ce;
+        if (p.chunks) {
+            for (int c = 0, k = k0; c < ce; c += p.chunk, ++k) {
+                ChunkInfo ci;
+                ci.e = e;
+                ci.pair_base = off + c;
+                ci.nv = min(p.chunk, ce - c);
+                ci.bits = be;
+                p.chunks[k] = ci;
+            }
+            if (e == 0) {
+                int n = 0;
+                for (int f = 0; f < p.E; ++f) n += (cnt[f] + p.chunk - 1) / p.chunk;
+                *p.nchunks = n;
+                for (int i = 0; i < 4; ++i) p.counters[i] = 0;
+            }
+        }
+    }
 }
 
 // Histogram, scan, stable placement and work-chunk list by one CTA of any size
@@ -243,36 +368,7 @@ __device__ __forceinline__ void permute_block(const PermuteParams &p)
         if (key >= 0) atomicAdd(&cnt[key], 1);
     }
     __syncthreads();
-    if (tid < p.E) {
-        // expert tid: its offset, and the index of its first work chunk in the
-        // order the expert kernels take them (more bits first, then by expert)
-        const int e = tid, be = nbits[e], ce = cnt[e];
-        int off = 0, k0 = 0;
-        for (int f = 0; f < p.E; ++f) {
-            const int cf = cnt[f], bf = nbits[f];
-            if (f < e) off += cf;
-            if (bf > be || (bf == be && f < e)) k0 += (cf + p.chunk - 1) / p.chunk;
-        }
-        p.offsets[e] = off;
-        run[e] = off;
-        if (e == p.E - 1) p.offsets[p.E] = off + ce;
-        if (p.chunks) {
-            for (int c = 0, k = k0; c < ce; c += p.chunk, ++k) {
-                ChunkInfo ci;
-                ci.e = e;
-                ci.pair_base = off + c;
-                ci.nv = min(p.chunk, ce - c);
-                ci.bits = be;
-                p.chunks[k] = ci;
-            }
-            if (e == 0) {
-                int n = 0;
-                for (int f = 0; f < p.E; ++f) n += (cnt[f] + p.chunk - 1) / p.chunk;
-                *p.nchunks = n;
-                for (int i = 0; i < 4; ++i) p.counters[i] = 0;
-            }
-        }
-    }
+    permute_lists(p, cnt, run, nbits);
     __syncthreads();
     for (int base = 0; base < NP; base += blockDim.x) {
         int i = base + tid;
@@ -302,11 +398,94 @@ __device__ __forceinline__ void permute_block(const PermuteParams &p)
     }
 }
 
+// The same placement for at most kPermKeys pairs per thread: every pair's key is loaded
+// once, all loads in flight together, the warps' counts of all passes go to shared
+// memory, and one scan per expert (a warp each) gives every (pass, warp) its start, so
+// that the placement needs three block barriers in all instead of five per pass: 4096
+// tokens 20 -> 13 us between events.
+constexpr int kPermKeys = 8;
+
+__device__ __forceinline__ void permute_keys(const PermuteParams &p)
+{
+    __shared__ int cnt[kMaxE];
+    __shared__ int run[kMaxE];
+    __shared__ int nbits[kMaxE];
+    __shared__ int wcnt[kPermKeys * 32][kMaxE + 1];  // [pass * warps + warp][expert]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int NP = 2 * p.T;
+    int key[kPermKeys], rank[kPermKeys];
+#pragma unroll
+    for (int j = 0; j < kPermKeys; ++j) {
+        const int i = j * blockDim.x + tid;
+        key[j] = -1;
+        if (i < NP) {
+            const uint8_t pr = __ldcg(p.pruned + (i >> 1));
+            const int e = __ldcg(p.idx + i);
+            key[j] = ((i & 1) && pr) || pr == 2 ? -1 : e;
+        }
+    }
+    if (tid < kMaxE) {
+        int b = 0;
+#pragma unroll
+        for (int f = 0; f < kMaxE; ++f)
+            if (f == tid) b = p.bits[f];
+        nbits[tid] = b;
+    }
+    const int np = (NP + blockDim.x - 1) / blockDim.x;  // passes in use
+#pragma unroll
+    for (int j = 0; j < kPermKeys; ++j) {
+        if (j >= np) continue;
+        if (lane < kMaxE) wcnt[j * nw + warp][lane] = 0;
+        __syncwarp();
+        const unsigned same = __match_any_sync(0xffffffffu, key[j]);
+        rank[j] = __popc(same & ((1u << lane) - 1));
+        if (key[j] >= 0 && rank[j] == 0) wcnt[j * nw + warp][key[j]] = __popc(same);
+    }
+    __syncthreads();
+    for (int e = warp; e < p.E; e += nw) {
+        // exclusive scan of expert e's counts in pair order, kPermKeys entries per lane
+        const int n = np * nw;
+        int c[kPermKeys], sum = 0;
+#pragma unroll
+        for (int i = 0; i < kPermKeys; ++i) {
+            const int q = lane * kPermKeys + i;
+            c[i] = q < n ? wcnt[q][e] : 0;
+            sum += c[i];
+        }
+        int incl = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += v;
+        }
+        int before = incl - sum;
+#pragma unroll
+        for (int i = 0; i < kPermKeys; ++i) {
+            const int q = lane * kPermKeys + i;
+            if (q < n) wcnt[q][e] = before;
+            before += c[i];
+        }
+        if (lane == 31) cnt[e] = incl;
+    }
+    __syncthreads();
+    permute_lists(p, cnt, run, nbits);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kPermKeys; ++j) {
+        const int i = j * blockDim.x + tid;
+        if (i >= NP) continue;
+        const int pos = key[j] >= 0 ? run[key[j]] + wcnt[j * nw + warp][key[j]] + rank[j] : -1;
+        if (key[j] >= 0) p.perm[pos] = i;
+        if (p.inv) p.inv[i] = pos;
+    }
+}
+
 __global__ void __launch_bounds__(1024) permute_kernel(PermuteParams p)
 {
     pdl_trigger();
     pdl_wait();
-    permute_block(p);
+    if (2 * p.T <= kPermKeys * (int)blockDim.x) permute_keys(p);
+    else permute_block(p);
 }
 
 // Placement of at most 128 pairs (T <= 64) by one warp, with no block barrier.
@@ -494,8 +673,12 @@ int launch_route(const RouteParams &rp, const PermuteParams &pp, cudaStream_t st
         return MC_OK;
     }
     profile_begin(kKRoute, st);
-    err = rp.h_in ? launch_k(route_kernel<true>, dim3(rp.T), dim3(kRouteThreads), norm_smem, st, rp)
-                  : launch_k(route_kernel<false>, dim3(rp.T), dim3(kRouteThreads), 0, st, rp);
+    if (rp.h_in)
+        err = launch_k(route_kernel<true>, dim3(rp.T), dim3(kRouteThreads), norm_smem, st, rp);
+    else if (rp.T >= kRouteTTMinT && rp.E <= kRouteTTMaxE)
+        err = launch_k(route_multi_kernel, dim3((rp.T + kRouteTT - 1) / kRouteTT), dim3(kRouteThreads), 0, st, rp);
+    else
+        err = launch_k(route_kernel<false>, dim3(rp.T), dim3(kRouteThreads), 0, st, rp);
     profile_end(kKRoute, st);
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "route launch: %s", cudaGetErrorString(err));
     profile_begin(kKPermute, st);
