@@ -103,16 +103,30 @@ def _ptr(t):
     if t is None:
         return None
     if isinstance(t, np.ndarray):
-        return t.ctypes.data
+        return _np_ptr(t)
     return t.data_ptr()
 
 
+def _np_ptr(a):
+    # (a.ctypes builds a helper object on every access)
+    return a.__array_interface__["data"][0]
+
+
 def _stream():
+    """torch's current stream on the current device, as the integer that the C calls take.
+
+    The raw-handle query costs a fraction of a microsecond where building a
+    torch.cuda.Stream object costs about three; a torch without it takes the object."""
     import torch
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _bits(bits):
+    if type(bits) is np.ndarray and bits.dtype == np.int8 and bits.flags.c_contiguous:
+        return bits
     return np.ascontiguousarray(bits, dtype=np.int8)
 
 
@@ -258,18 +272,18 @@ def moe_forward(x, gate_w, shape: Shape, bits, packed_dev, mu: float = 0.0, prot
     """The whole layer.  x bf16 [T,H]; returns y bf16 [T,H] (and routing tensors)."""
     import torch
     T = x.shape[0]
-    dev = x.device
     if y is None:
         y = torch.empty_like(x)
     if workspace is None:
-        workspace = alloc_workspace(shape, T, dev)
+        workspace = alloc_workspace(shape, T, x.device)
     b = _bits(bits)
     idx = w = pr = None
     if routing:
+        dev = x.device
         idx = torch.empty((T, 2), dtype=torch.int32, device=dev)
         w = torch.empty((T, 2), dtype=torch.float32, device=dev)
         pr = torch.empty(T, dtype=torch.uint8, device=dev)
-    _check(load().mc_moe_forward(_ptr(x), _ptr(gate_w), T, ctypes.byref(shape), b.ctypes.data, _ptr(packed_dev),
+    _check(load().mc_moe_forward(_ptr(x), _ptr(gate_w), T, ctypes.byref(shape), _np_ptr(b), _ptr(packed_dev),
                                  float(mu), _ptr(protect), _ptr(y), _ptr(workspace), workspace.numel(),
                                  _ptr(idx), _ptr(w), _ptr(pr), _stream()))
     if routing:
@@ -288,7 +302,7 @@ def moe_forward_static(x, gate_w, shape: Shape, bits, packed_dev, mu: float = 0.
     if y is None:
         y = torch.empty_like(x)
     b = _bits(bits)
-    _check(load().mc_moe_forward_static(_ptr(x), _ptr(gate_w), T, ctypes.byref(shape), b.ctypes.data,
+    _check(load().mc_moe_forward_static(_ptr(x), _ptr(gate_w), T, ctypes.byref(shape), _np_ptr(b),
                                         _ptr(packed_dev), float(mu), _ptr(protect), _ptr(y), _ptr(status),
                                         _stream()))
     return y
@@ -319,8 +333,8 @@ def stack_forward(h, shape: Shape, args: StackArgs, gamma, workspace, protect=No
     """mc_stack_forward: h (bf16 [T,H], device) updated in place."""
     T = h.shape[0]
     _check(load().mc_stack_forward(_ptr(h), T, ctypes.byref(shape), args.layers,
-                                   ctypes.cast(args.gate_ptrs, ctypes.c_void_p), args.bits.ctypes.data,
-                                   ctypes.cast(args.packed_ptrs, ctypes.c_void_p), args.mus.ctypes.data,
+                                   ctypes.addressof(args.gate_ptrs), _np_ptr(args.bits),
+                                   ctypes.addressof(args.packed_ptrs), _np_ptr(args.mus),
                                    _ptr(protect), _ptr(gamma), float(eps), _ptr(workspace), workspace.numel(),
                                    _stream()))
     return h
