@@ -142,8 +142,10 @@ inline cudaError_t launch_k(void (*kernel)(P...), dim3 grid, dim3 block, size_t 
 
 // Host launchers: MC_OK or an MC_ERR_* code with the message set.
 // done: a zeroed device counter enabling the single-launch routing + placement for
-// T <= 64 (left at zero), or NULL for two launches.
-int launch_route(const RouteParams &rp, const PermuteParams &pp, cudaStream_t st, int32_t *done = nullptr);
+// T <= 64 (left at zero), or NULL for two launches; cluster: take the single cluster
+// launch for T <= 16, which needs no counter, even without one.
+int launch_route(const RouteParams &rp, const PermuteParams &pp, cudaStream_t st, int32_t *done = nullptr,
+                 bool cluster = false);
 int launch_gemv(ExpertParams ep, cudaStream_t st);   // mma.sync path
 int launch_gemm(ExpertParams ep, cudaStream_t st);   // prefill path (tcgen05 grouped GEMM)
 size_t img_buffer_bytes(int max_blocks, int cols);

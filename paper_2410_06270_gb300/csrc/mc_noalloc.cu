@@ -157,7 +157,9 @@ extern "C" int mc_moe_forward_static(const void *x, const void *gate_w, int T, c
     pp.nchunks = ws.nchunks;
     pp.counters = ws.counters;
     pp.chunk = kChunk;
-    if ((rc = launch_route(rp, pp, st))) return rc;
+    // up to 16 tokens in one cluster launch, which needs no zeroed word (the scratch has
+    // none); above them the routing and the placement are two launches
+    if ((rc = launch_route(rp, pp, st, nullptr, true))) return rc;
 
     ExpertParams ep{};
     memset(&ep, 0, sizeof ep);  // the tensor-core path's buffers stay NULL: not used here

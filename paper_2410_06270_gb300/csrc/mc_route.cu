@@ -480,14 +480,6 @@ __device__ __forceinline__ void permute_keys(const PermuteParams &p)
     }
 }
 
-__global__ void __launch_bounds__(1024) permute_kernel(PermuteParams p)
-{
-    pdl_trigger();
-    pdl_wait();
-    if (2 * p.T <= kPermKeys * (int)blockDim.x) permute_keys(p);
-    else permute_block(p);
-}
-
 // Placement of at most 128 pairs (T <= 64) by one warp, with no block barrier.
 // Pair i = 32k + lane sits in slice k.  Lane e (< E) keeps, per slice, the ballot
 // of the lanes whose pair goes to expert e; their population counts give the
@@ -496,6 +488,8 @@ __global__ void __launch_bounds__(1024) permute_kernel(PermuteParams p)
 // it in the slice.  Same result as permute_block.
 //   dec (optional): the tokens' decisions in shared memory (e0, e1, pruned at 3 t)
 //   instead of the routing outputs in global memory.
+constexpr int kPermWarpMaxT = 64;
+
 __device__ __forceinline__ void permute_warp(const PermuteParams &p, const int *dec = nullptr)
 {
     const unsigned full = 0xffffffffu, lt = (1u << (threadIdx.x & 31)) - 1;
@@ -570,6 +564,15 @@ __device__ __forceinline__ void permute_warp(const PermuteParams &p, const int *
             if (p.inv && i < NP) p.inv[i] = pos;
             start += __popc(mine[k]);
         }
+}
+
+__global__ void __launch_bounds__(1024) permute_kernel(PermuteParams p)
+{
+    pdl_trigger();
+    pdl_wait();
+    if (p.T <= kPermWarpMaxT) permute_warp(p);  // one warp
+    else if (2 * p.T <= kPermKeys * (int)blockDim.x) permute_keys(p);
+    else permute_block(p);
 }
 
 // Routing of token blockIdx.x, then the last CTA to finish (counted on *done,
@@ -652,12 +655,12 @@ static cudaError_t launch_route_cluster(const RouteParams &rp, const PermutePara
     return cudaLaunchKernelEx(&cfg, route_cluster_kernel<NORM>, rp, pp);
 }
 
-int launch_route(const RouteParams &rp, const PermuteParams &pp, cudaStream_t st, int32_t *done)
+int launch_route(const RouteParams &rp, const PermuteParams &pp, cudaStream_t st, int32_t *done, bool cluster)
 {
     // the pre-norm row (mc_stack_forward's layers) in dynamic shared memory
     const size_t norm_smem = rp.h_in ? (size_t)rp.H * 2 : 0;
     cudaError_t err;
-    if (done && rp.T <= kClusterMaxT) {
+    if ((done || cluster) && rp.T <= kClusterMaxT) {
         profile_begin(kKRoute, st);
         err = rp.h_in ? launch_route_cluster<true>(rp, pp, norm_smem, st) : launch_route_cluster<false>(rp, pp, 0, st);
         profile_end(kKRoute, st);
@@ -682,8 +685,8 @@ int launch_route(const RouteParams &rp, const PermuteParams &pp, cudaStream_t st
     profile_end(kKRoute, st);
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "route launch: %s", cudaGetErrorString(err));
     profile_begin(kKPermute, st);
-    // one thread per pair (whole warps), at most 1024: fewer threads to synchronise for small T
-    const int nt = min(1024, max(32, (2 * pp.T + 31) / 32 * 32));
+    // one warp for few pairs, then one thread per pair (whole warps), at most 1024
+    const int nt = pp.T <= kPermWarpMaxT ? 32 : min(1024, (2 * pp.T + 31) / 32 * 32);
     err = launch_k(permute_kernel, dim3(1), dim3(nt), 0, st, pp);
     profile_end(kKPermute, st);
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "permute launch: %s", cudaGetErrorString(err));
