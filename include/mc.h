@@ -193,7 +193,8 @@ int mc_moe_forward(const void *x, const void *gate_w, int T, const mc_shape *sha
  *     more than 16 MiB returns MC_ERR_INVALID_ARG with the size in the message
  *     (at the Mixtral-8x7b shape, H 4096, F 14336, group 128, that is T > 96).
  *     The W2 pass takes mc_moe_forward's column splits when their partial
- *     outputs fit in the scratch, else a single split (same results).
+ *     outputs fit in the scratch, else fewer (same results but for the order of
+ *     fp32 sums).
  *   Set-up: the first call on a device, made with that device current, looks up
  *     the scratch's address once (cudaGetSymbolAddress) and keeps it for the
  *     life of the process; make that first call before any stream capture, and

@@ -33,17 +33,26 @@ static std::atomic<unsigned long long> g_timeout_ns{1000000000ull};  // 1 s
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Column splits of the W2 GEMV pass.  The workspace holds up to kMaxKS splits
+// Column splits of the W2 GEMV pass.  The workspace holds up to max_ks splits
 // (decode sizes); the forward picks, among the divisors of F/128 that leave each
 // item at least two ring stages, the split count whose work items (estimated
 // chunks x 256-row block pairs x splits) fill the SMs' last wave best, the
-// smaller one on ties.
+// smaller one on ties.  Above 64 tokens the chunk count depends on how the pairs fall,
+// so the most splits are taken: many short items leave a short last wave whatever it
+// is (Mixtral-8x7b layer, W2 launch without splits -> with 7: 65 tokens 112 -> 74 us,
+// 80: 112 -> 88, 96: 112 -> 98, 112: 112 -> 103; the layer 252 -> 218, 279 -> 258, 300 ->
+// 289, 310 -> 305).
 
-int max_ks(const mc_shape *s, int T) { return T > 64 ? 1 : kMaxKS; }
+int max_ks(const mc_shape *s, int T) { return 2 * T < kPrefillPairs ? kMaxKS : 1; }
 
 int choose_ks(const mc_shape *s, int T, int nsm)
 {
     const int nt = s->F / kTileK, npairs = (s->H / kBlockRows + 1) / 2;
+    if (T > 64) {
+        int ks = max_ks(s, T);
+        while (ks > 1 && (nt % ks || nt / ks < 8)) --ks;
+        return ks;
+    }
     const int chunks = 2 * T < s->E ? 2 * T : s->E;  // pairs land on distinct experts at small T
     int best = 1;
     double best_eff = -1.0;

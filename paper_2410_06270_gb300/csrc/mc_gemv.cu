@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) gemv_pp_kernel(ExpertParams p)
 // with a residual (the pre-norm stack), y[t] = resid[t] + that, rounded to bf16
 // first (the layer's own output) and once more after the fp32 add.
 //
-// A single split (the GEMM, and the GEMV above 64 tokens): both slots' rows loaded
+// A single split (the GEMM, and the GEMV above 64 tokens when it takes one): both slots' rows loaded
 // at once, 4 columns per thread, no per-split registers, so that enough loads are in
 // flight to stream the partial outputs: 71 -> 30 us between events at 4096 tokens (134
 // MB in, 33 MB out; 8 columns per thread, slot by slot, before).
@@ -996,7 +996,7 @@ __global__ void __launch_bounds__(256) combine1_kernel(CombineParams p)
     *reinterpret_cast<uint2 *>(p.y + (size_t)t * p.H + c) = *reinterpret_cast<uint2 *>(r);
 }
 
-// The same for decode-sized calls (T <= 64), whose W2 pass may be split: one thread
+// The same for decode-sized calls, whose W2 pass may be split: one thread
 // per 4 output columns in 128-thread CTAs, so that the grid spreads over the SMs, and
 // every split of both slots loaded before the first is used (one round trip after the
 // routing outputs).
@@ -1125,12 +1125,10 @@ int launch_combine(const CombineParams &cp, cudaStream_t st)
     if (cp.KS < 1 || cp.KS > kMaxKS) return set_error(MC_ERR_INVALID_ARG, "combine: %d column splits", cp.KS);
     profile_begin(kKCombine, st);
     cudaError_t err;
-    if (cp.T <= kCombine4MaxT) {
+    if (cp.KS > 1 || cp.T <= kCombine4MaxT) {
         const int n = cp.T * (cp.H / 4);
         err = launch_k(combine4_kernel, dim3((n + 127) / 128), dim3(128), 0, st, cp);
     } else {
-        // (max_ks: one split above 64 tokens)
-        if (cp.KS != 1) return set_error(MC_ERR_INVALID_ARG, "combine: %d column splits for %d tokens", cp.KS, cp.T);
         const int n = cp.T * (cp.H / 4);
         err = launch_k(combine1_kernel, dim3((n + 255) / 256), dim3(256), 0, st, cp);
     }

@@ -106,14 +106,16 @@ extern "C" int mc_moe_forward_static(const void *x, const void *gate_w, int T, c
         (status_dev && !aligned(status_dev, 4)))
         return set_error(MC_ERR_INVALID_ARG, "x, gate_w, y need 16-byte and packed_dev 256-byte alignment");
     // W2 column splits: mc_moe_forward's choice when its partial outputs fit in
-    // the scratch, else a single split (the limit below is the single split's)
+    // the scratch, else fewer (the limit below is the single split's)
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return set_error(MC_ERR_CUDA, "device query failed");
     int KS = choose_ks(shape, T, nsm);
     size_t need = carve_static(shape, T, KS, nullptr).total;
-    if (need > kStaticScratchBytes && KS > 1) {
-        KS = 1;
+    const int nt = shape->F / kTileK;
+    while (need > kStaticScratchBytes && KS > 1) {  // the most splits that fit
+        do --KS;
+        while (nt % KS);
         need = carve_static(shape, T, KS, nullptr).total;
     }
     if (need > kStaticScratchBytes)

@@ -215,6 +215,15 @@ def test_forward_bit_widths_and_groups(mc, bits, group):
     _forward_and_check(mc, L)
 
 
+@pytest.mark.parametrize("T", [64, 65, 119, 120])
+def test_forward_w2_column_splits(mc, T):
+    """Both sides of the limits of the W2 GEMV pass's column splits (F of 16 and more
+    column steps, so that splits exist), on the GEMV path."""
+    L = synth.make_layer(T, 512, 4096, 8, 128, [3, 2, 1, 3, 2, 2, 1, 3], 980 + T, gate_std=0.05, mu=0.2,
+                         protect_frac=0.2)
+    _forward_and_check(mc, L, tokens=[0, 1, T // 2, T - 1], path=1)
+
+
 def test_forward_fractional_zeros(mc):
     """Arbitrary fp16 zero points (HQQ-style storage), not only integer ones."""
     L = synth.make_layer(16, 384, 640, 8, 128, [3, 2, 1, 2, 3, 2, 1, 3], 70, gate_std=0.1,
