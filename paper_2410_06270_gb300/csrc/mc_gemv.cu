@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(ExpertParams p)
 constexpr int kPPKPS = 2;                  // 128-column steps per stage
 constexpr int kPPSlots = 2;                // ring slots per group
 constexpr int kPPThreads = 2 * (kCW + 1) * 32;
-constexpr int kPPMinPairs = 32;            // 2 T from which a quantised layer takes this kernel
+constexpr int kPPMinPairs = 20;            // 2 T from which a quantised layer takes this kernel
 
 struct PPGroup {
     uint64_t full[kPPSlots], empty[kPPSlots];
@@ -1060,10 +1060,10 @@ int launch_gemv(ExpertParams ep, cudaStream_t st)
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "device query: %s", cudaGetErrorString(err));
     // 16-bit experts are all or none of a layer (check_bits).  Quantised layers of
-    // >= 16 tokens run the two-group kernel: measured on the Mixtral-8x7b layer at
-    // 16 tokens 127.9 K against 120.8 K tokens/s; at 1 and 4 tokens it was slower
-    // (15.3 / 33.2 K against 17.2 / 36.3 K: with about one item per SM one group
-    // idles and the other's two-slot ring is too shallow to keep the stream busy)
+    // >= 10 tokens run the two-group kernel.  Mixtral-8x7b layer, one group / two groups:
+    // 5 tokens 113.1 / 114.3 us, 8: 114.8 / 115.4, 9: 120.9 / 117.4, 12: 122.1 / 117.2, 15:
+    // 122.1 / 117.9 (with about one item per SM one group idles and the other's two-slot
+    // ring is too shallow to keep the stream busy: 1 token 58 / 65 us when it was measured)
     const bool dense = ep.bits[0] == 16;
     if (!dense && ep.Pmax >= kPPMinPairs) {
         const size_t smp = pp_smem(ep.group);
