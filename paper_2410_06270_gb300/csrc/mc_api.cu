@@ -16,10 +16,13 @@ namespace mc {
 // expert paths of mc_moe_forward (mc_set_path)
 constexpr int kPathAuto = 0, kPathGemv = 1, kPathGemm = 2;
 static std::atomic<int> g_path{kPathAuto};
-// pairs (2 T) from which mc_moe_forward's automatic choice is the prefill GEMM:
-// measured on the Mixtral-8x7b layer, the GEMV path (each weight tile decoded
-// once per 16-pair chunk) is faster up to ~96 tokens, the GEMM (once per
-// 128-pair token block) from ~128 tokens on
+// pairs (2 T) from which mc_moe_forward's automatic choice is the prefill GEMM.
+// Mixtral-8x7b layer, GEMV (each weight tile decoded once per 16-pair chunk) / GEMM
+// (once per 128-pair token block): 32 tokens 149 / 195 us, 64: 214 / 199, 80: 257 /
+// 203, 96: 288 / 206, 119: 334 / 206, 128: 383 / 208.  The line lies above the
+// crossover in time (~60 tokens) because the GEMM multiplies weights rounded to fp16
+// and the GEMV path exact codes: relative error of the layer output against 64 bits
+// 1.9e-3 and 1.7e-3.  A lower line would lose precision between the two.
 constexpr int kPrefillPairs = 240;
 static std::atomic<int> g_debug{0};
 static std::atomic<unsigned long long> g_timeout_ns{1000000000ull};  // 1 s
