@@ -36,8 +36,10 @@ static std::atomic<unsigned long long> g_timeout_ns{1000000000ull};  // 1 s
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Column splits of the W2 GEMV pass.  The workspace holds up to max_ks splits
-// (decode sizes); the forward picks, among the divisors of F/128 that leave each
+// Column splits of the W2 GEMV pass.  The workspace holds up to max_ks splits: the
+// kMaxKS of decode sizes have room of their own; from 65 tokens the partial outputs lie
+// over the GEMM's image buffers, which a GEMV call does not use, so the workspace is no
+// larger than the GEMM needs and one of more tokens serves every T.  The forward picks, among the divisors of F/128 that leave each
 // item at least two ring stages, the split count whose work items (estimated
 // chunks x 256-row block pairs x splits) fill the SMs' last wave best, the
 // smaller one on ties.  Above 64 tokens the chunk count depends on how the pairs fall,
@@ -46,7 +48,19 @@ static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // 80: 112 -> 88, 96: 112 -> 98, 112: 112 -> 103; the layer 252 -> 218, 279 -> 258, 300 ->
 // 289, 310 -> 305).
 
-int max_ks(const mc_shape *s, int T) { return 2 * T < kPrefillPairs ? kMaxKS : 1; }
+static size_t image_bytes(const mc_shape *s, int T)
+{
+    const int nb = max_blocks_for(T, s->E);
+    return align256(img_buffer_bytes(nb, s->H)) + align256(img_buffer_bytes(nb, s->F));
+}
+
+int max_ks(const mc_shape *s, int T)
+{
+    if (T <= 64) return kMaxKS;
+    if (2 * T >= kPrefillPairs) return 1;
+    const size_t fit = 1 + image_bytes(s, T) / ((size_t)2 * T * s->H * 4);  // images + one split's room
+    return fit < (size_t)kMaxKS ? (int)fit : kMaxKS;
+}
 
 int choose_ks(const mc_shape *s, int T, int nsm)
 {
@@ -82,8 +96,9 @@ struct Workspace {
     int32_t *route_done;  // zero between calls: single-launch routing for small T
     uint8_t *xvec, *hvec;
     uint8_t *ximg, *himg;
-    float *opart;
-    int max_chunks, max_blocks, KS;
+    float *opart;        // W2 outputs of the GEMM
+    float *opart_split;  // of the GEMV, max_ks column splits
+    int max_chunks, max_blocks;
     size_t total;
 };
 
@@ -97,7 +112,6 @@ static Workspace carve(const mc_shape *s, int T, void *base)
         off = align256(off + bytes);
         return r;
     };
-    w.KS = max_ks(s, T);  // room for the largest split count the forward may pick
     w.max_chunks = max_chunks_for(T, s->E);
     const size_t P = 2 * (size_t)T, MC = (size_t)w.max_chunks;
     // The words that must be zero when a call starts (and that every call leaves
@@ -119,7 +133,8 @@ static Workspace carve(const mc_shape *s, int T, void *base)
     w.max_blocks = max_blocks_for(T, s->E);
     w.ximg = (uint8_t *)take(img_buffer_bytes(w.max_blocks, s->H));
     w.himg = (uint8_t *)take(img_buffer_bytes(w.max_blocks, s->F));
-    w.opart = (float *)take((size_t)w.KS * P * s->H * 4);
+    w.opart = (float *)take((size_t)(T > 64 ? 1 : kMaxKS) * P * s->H * 4);
+    w.opart_split = T > 64 ? (float *)w.ximg : w.opart;  // max_ks splits end where opart does
     w.total = off;
     return w;
 }
@@ -307,7 +322,7 @@ int mc::moe_forward_ex(const void *x, const void *gate_w, int T, const mc_shape 
     ep.ximg = ws.ximg;
     ep.himg = ws.himg;
     ep.max_blocks = ws.max_blocks;
-    ep.opart = ws.opart;
+    ep.opart = path == kPathGemm ? ws.opart : ws.opart_split;
     int nsm = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return set_error(MC_ERR_CUDA, "device query failed");
@@ -322,7 +337,7 @@ int mc::moe_forward_ex(const void *x, const void *gate_w, int T, const mc_shape 
     if (rc) return rc;
 
     CombineParams cp{};
-    cp.opart = ws.opart;
+    cp.opart = ep.opart;
     cp.w = ws.w;
     cp.inv = ws.inv;
     cp.T = T;

@@ -159,6 +159,15 @@ def test_workspace_size_grows_with_tokens(mc):
     assert 0 < a < b
 
 
+@pytest.mark.parametrize("dims", [(8, 4096, 14336, 128), (8, 6144, 16384, 128), (2, 1024, 1024, 64), (4, 2048, 256, 64)])
+def test_workspace_of_more_tokens_covers_fewer(mc, dims):
+    """A workspace sized for any T_max >= 65 covers every T from 65 up to it, across the
+    limit between the GEMV with column splits and the GEMM."""
+    s = mc.Shape(*dims)
+    sizes = [mc.workspace_size(s, T) for T in range(65, 301)]
+    assert sizes == sorted(sizes)
+
+
 def test_odp_threshold_host_matches_oracle():
     """mc_odp_threshold_host (host code, no GPU) against the oracle's quantile of
     w1/w0 over the prunable tokens."""

@@ -224,6 +224,23 @@ def test_forward_w2_column_splits(mc, T):
     _forward_and_check(mc, L, tokens=[0, 1, T // 2, T - 1], path=1)
 
 
+@pytest.mark.parametrize("E,H,F", [(8, 512, 4096), (2, 4096, 2048)])
+def test_one_workspace_across_the_gemm_limit(mc, E, H, F):
+    """A workspace of 130 tokens (GEMM) serves 119, 65 and 100 tokens (W2 column splits,
+    whose partial outputs lie over the GEMM's images) and again 130, each bit for bit
+    as with a workspace of its own."""
+    shape = mc.Shape(E, H, F, 128)
+    ws = mc.alloc_workspace(shape, 130)
+    for T in (119, 130, 65, 100, 130):
+        L = synth.make_layer(T, H, F, E, 128, ([3, 2, 1, 3, 2, 2, 1, 3])[:E], 990 + T, gate_std=0.05)
+        shape, packed = _pack(mc, L)
+        x, g, p = to_dev(L)
+        y = mc.moe_forward(x, g, shape, L.bits, packed, L.mu, p, workspace=ws)
+        y_own = mc.moe_forward(x, g, shape, L.bits, packed, L.mu, p)
+        mc.check_status(ws)
+        assert torch.equal(y, y_own), "T=%d" % T
+
+
 def test_forward_fractional_zeros(mc):
     """Arbitrary fp16 zero points (HQQ-style storage), not only integer ones."""
     L = synth.make_layer(16, 384, 640, 8, 128, [3, 2, 1, 2, 3, 2, 1, 3], 70, gate_std=0.1,
