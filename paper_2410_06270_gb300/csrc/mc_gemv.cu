@@ -46,8 +46,8 @@ struct RingShared {
     uint64_t cbar;  // consumer-warp barrier of the W13 epilogue (bounded waits)
     volatile int abort;
     volatile int issued;
+    volatile int stopped;  // the producer left on an abort: it takes no slot any more
     int slot_item[kMaxSlots];
-    int slot_kc[kMaxSlots];  // column steps held by the stage (1..kKPS)
     ChunkInfo slot_ci[kMaxSlots];  // the stage's chunk
 };
 static_assert(256 + sizeof(RingShared) <= 1024, "ring header");
@@ -77,8 +77,8 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, co
     if (mbar_try_wait(bar, parity)) return true;
     uint64_t t0 = globaltimer_ns();
     while (true) {
-        if (mbar_try_wait_sleep(bar, parity, kWaitHintNs)) return true;
         if (*abort) return false;
+        if (mbar_try_wait_sleep(bar, parity, kWaitHintNs)) return true;
         if (globaltimer_ns() - t0 > p.timeout_ns) {
             set_status(p.status, MC_ERR_TIMEOUT);
             *abort = 1;
@@ -86,9 +86,17 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, co
         }
     }
 }
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, const ExpertParams &p, RingShared *sh)
+
+// A whole warp's wait, with one answer for all of its lanes: what follows such a
+// wait is executed by the warp together (mma.sync, __syncwarp), and lanes that took
+// different answers, when a phase completes just as a wait expires or the CTA aborts,
+// would wait for one another for ever.  False also where the CTA had aborted before the
+// wait (read ahead of it, so that the read costs no time): a warp that went through an
+// item after an abort ends there, whatever the parity of the slot it has come to.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, const ExpertParams &p, volatile int *abort)
 {
-    return wait_or_abort(bar, parity, p, &sh->abort);
+    const bool live = !*abort;
+    return __all_sync(0xffffffffu, wait_or_abort(bar, parity, p, abort) && live);
 }
 
 // The packed buffer must carry the header written for this shape and bit table:
@@ -441,13 +449,11 @@ struct Ring {
     const uint2 *afr;  // A fragments of the table matrix
 };
 
-// What one group of consumer warps shares: the CTA's abort flag, the group's
-// epilogue barrier, the column steps of each of its ring's stages, and the
-// thread's index within the group.
+// What one group of consumer warps shares: the CTA's abort flag, its producer's
+// stopped flag, the group's epilogue barrier, and the thread's index within the group.
 struct GroupCtx {
-    volatile int *abort;
+    volatile int *abort, *stopped;
     uint64_t *cbar;
-    const int *slot_kc;
     int gtid;
 };
 
@@ -457,7 +463,28 @@ __device__ __forceinline__ bool consumer_sync(const ExpertParams &p, const Group
 {
     __syncwarp();
     if (lane == 0) mbar_arrive(G.cbar);
-    return wait_or_abort(G.cbar, (uses++) & 1, p, G.abort);
+    return warp_wait(G.cbar, (uses++) & 1, p, G.abort);
+}
+
+// A consumer warp's wait between an item's stages.  It answers nothing, so that every lane
+// goes through all of the item whatever its own wait came to (each mma.sync waits for the
+// whole warp), on whatever the slot holds if the CTA has aborted; the warp leaves at the
+// next wait that it votes on.  After an abort a lane goes on only once the producer has
+// stopped: the slots that it gives back from then on were not filled again.
+//   A vote after every stage's wait instead, with an exit from the loop: the Mixtral-8x7b
+// layer at 16 / 64 tokens 115.4 / 211 -> 117.5 / 215 us; this form 114.7 / 211.
+__device__ __forceinline__ void wait_in_item(uint64_t *bar, uint32_t parity, const ExpertParams &p, const GroupCtx &G)
+{
+    if (mbar_try_wait(bar, parity)) return;
+    const uint64_t t0 = globaltimer_ns();
+    while (!mbar_try_wait_sleep(bar, parity, kWaitHintNs)) {
+        if (*G.stopped) return;
+        if (globaltimer_ns() - t0 > p.timeout_ns) {
+            set_status(p.status, MC_ERR_TIMEOUT);
+            *G.abort = 1;
+            return;
+        }
+    }
 }
 
 // One work item for one consumer warp: all its stages, then the epilogue.  The
@@ -488,9 +515,12 @@ __device__ __forceinline__ bool run_item(const ExpertParams &p, const GroupCtx &
 #pragma unroll
             for (int c = 0; c < 4; ++c) y[u][j][c] = 0.f;
     for (int i = 0; i < I.nkt; i += KPS) {
-        if (i > 0 && !wait_or_abort(&R.full[slot], phase, p, G.abort)) return false;
+        if (i > 0) wait_in_item(&R.full[slot], phase, p, G);
         const uint8_t *base = R.base + (size_t)slot * R.SB;
-        const int kc = G.slot_kc[slot];
+        // the stage's column steps, the same in every lane by construction; the empty asm
+        // keeps the compiler from reshaping the loop around it (16 tokens 116.6 -> 114.7 us)
+        int kc = min(KPS, I.nkt - i);
+        asm volatile("" : "+r"(kc));
         const uint8_t *v0 = base + R.vec_off0, *v1 = v0 + KPS * R.VB;
         auto step = [&](int kk) {
             const uint8_t *st = base + kk * step_bytes;
@@ -590,6 +620,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(ExpertParams p)
         mbar_init(&sh->cbar, kCW);
         sh->abort = 0;
         sh->issued = 0;
+        sh->stopped = 0;
         fence_mbar_init();
     }
     if (W13) build_tab_afrag(afr, threadIdx.x, kGemvThreads);
@@ -644,7 +675,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(ExpertParams p)
                     p.packed + p.mat_off[e][W13 ? 0 : 2] + supertile_off(W13 ? 0 : 2, I.blkA, I.kt0, KTm, nrb, STB);
                 for (int i = 0, st = 0; i < I.nkt; i += KPS, ++it, ++st) {
                     const int slot = pslot;
-                    if (it >= S && !wait_or_abort(&empty[slot], pphase ^ 1u, p, sh)) {
+                    if (it >= S && !wait_or_abort(&empty[slot], pphase ^ 1u, p, &sh->abort)) {
                         ok = false;
                         break;
                     }
@@ -655,7 +686,6 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(ExpertParams p)
                     const int kc = min(KPS, I.nkt - i);
                     sh->slot_item[slot] = item;
                     sh->slot_ci[slot] = I.ci;
-                    sh->slot_kc[slot] = kc;
                     uint8_t *dst = ring + (size_t)slot * SB;
                     const uint32_t wb = (uint32_t)(kc * pw * STB), vb = (uint32_t)(kc * VB);
                     mbar_arrive_expect_tx(&full[slot], wb + NT * vb);
@@ -681,21 +711,22 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(ExpertParams p)
             if (ok) {
                 // end marker: one more stage with item -1 and no data
                 const int slot = pslot;
-                if (it < S || wait_or_abort(&empty[slot], pphase ^ 1u, p, sh)) {
+                if (it < S || wait_or_abort(&empty[slot], pphase ^ 1u, p, &sh->abort)) {
                     sh->slot_item[slot] = -1;
                     mbar_arrive(&full[slot]);
                 }
             }
         }
+        if (lane == 0 && sh->abort) sh->stopped = 1;
     } else {
         // --------------------------------------------------------- consumers --
         const Ring R{full, empty, ring, S, SB, vec_off0, VB, afr};
-        const GroupCtx G{&sh->abort, &sh->cbar, sh->slot_kc, (int)threadIdx.x};
+        const GroupCtx G{&sh->abort, &sh->stopped, &sh->cbar, (int)threadIdx.x};
         const int tl = warp;
         int slot = 0, items = 0, cbar_uses = 0;
         uint32_t phase = 0;
         while (true) {
-            if (!wait_or_abort(&full[slot], phase, p, sh)) break;
+            if (!warp_wait(&full[slot], phase, p, &sh->abort)) break;
             const int item = sh->slot_item[slot];
             if (item < 0) break;
             const Item I = decode_item<W13>(p, item, U, sh->slot_ci[slot]);
@@ -746,7 +777,8 @@ struct PPGroup {
     uint64_t full[kPPSlots], empty[kPPSlots];
     uint64_t cbar;
     volatile int issued;
-    int slot_item[kPPSlots], slot_kc[kPPSlots];
+    volatile int stopped;  // the producer left on an abort: it takes no slot any more
+    int slot_item[kPPSlots];
     ChunkInfo slot_ci[kPPSlots];
 };
 struct PPShared {
@@ -812,7 +844,6 @@ __device__ __forceinline__ void pp_produce(const ExpertParams &p, PPShared *sh, 
             const int kc = min(kPPKPS, I.nkt - i);
             G.slot_item[slot] = item;
             G.slot_ci[slot] = I.ci;
-            G.slot_kc[slot] = kc;
             uint8_t *dst = ring + (size_t)slot * SB;
             const uint32_t wb = (uint32_t)(kc * pw * STB), vb = (uint32_t)(kc * VB);
             mbar_arrive_expect_tx(&G.full[slot], wb + NT * vb);
@@ -869,6 +900,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) gemv_pp_kernel(ExpertParams p)
             }
             mbar_init(&sh->g[gg].cbar, kCW);
             sh->g[gg].issued = 0;
+            sh->g[gg].stopped = 0;
         }
         sh->abort = 0;
         sh->producers_done = 0;
@@ -905,15 +937,16 @@ __global__ void __launch_bounds__(kPPThreads, 1) gemv_pp_kernel(ExpertParams p)
                 pp_produce<W13>(p, sh, G, ring, SB, VB, vec_off0, item, ci, total, U, nrb, KTm, vbase, counter);
             }
         }
+        if (lane == 0 && sh->abort) G.stopped = 1;
     } else {
         // --------------------------------------------------------- consumers --
         const Ring R{G.full, G.empty, ring, kPPSlots, SB, vec_off0, VB, afr};
-        const GroupCtx Gc{&sh->abort, &G.cbar, G.slot_kc, lw * 32 + lane};
+        const GroupCtx Gc{&sh->abort, &G.stopped, &G.cbar, lw * 32 + lane};
         const int tl = lw;
         int slot = 0, items = 0, cbar_uses = 0;
         uint32_t phase = 0;
         while (true) {
-            if (!wait_or_abort(&G.full[slot], phase, p, &sh->abort)) break;
+            if (!warp_wait(&G.full[slot], phase, p, &sh->abort)) break;
             const int it_id = G.slot_item[slot];
             if (it_id < 0) break;
             const Item I = decode_item<W13>(p, it_id, U, G.slot_ci[slot]);

@@ -49,7 +49,8 @@ __global__ void __launch_bounds__(128) selftest_umma_kernel(const __half *A, con
         }
         umma_commit(bar);
     }
-    const bool ok = mbar_wait(bar, 0, timeout_ns, status);
+    // (one answer per warp: the loads below are executed by the warp together)
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, 0, timeout_ns, status));
     tc_fence_after();
     if (ok) {
         for (int c0 = 0; c0 < N; c0 += 16) {
@@ -108,7 +109,8 @@ __global__ void __launch_bounds__(128) selftest_umma_ts_kernel(const __half *A, 
         }
         umma_commit(bar);
     }
-    const bool ok = mbar_wait(bar, 0, timeout_ns, status);
+    // (one answer per warp: the loads below are executed by the warp together)
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, 0, timeout_ns, status));
     tc_fence_after();
     if (ok) {
         for (int c0 = 0; c0 < N; c0 += 16) {

@@ -91,6 +91,34 @@ def test_automatic_switch_agrees_with_gemv(mc):
     assert_close(auto, gemv.astype(np.float64), "automatic vs GEMV")
 
 
+def test_bounded_wait_reports_timeout_and_context_survives(mc):
+    """With the weight producer starved every wait of both GEMM launches runs out: the
+    call returns, the status word says so, and the next call is right again."""
+    L = synth.make_layer(300, 256, 384, 8, 64, [3, 2, 1, 3, 2, 2, 1, 3], 360, gate_std=0.1)
+    condition_routing(L)
+    shape = mc.Shape(L.E, L.H, L.F, L.group)
+    packed = mc.pack_experts(shape, L.bits, flat(L, "codes"), flat(L, "scale"), flat(L, "zero"))
+    x, g, p = to_dev(L)
+    ws = mc.alloc_workspace(shape, L.T)
+    old = mc.set_path(PATH_GEMM)
+    try:
+        mc.set_debug(1, 20_000_000)  # the producer issues nothing; waits give up after 20 ms
+        try:
+            mc.moe_forward(x, g, shape, L.bits, packed, workspace=ws)
+            with pytest.raises(mc.MCError) as ei:
+                mc.check_status(ws)
+            assert ei.value.code == mc.ERR_TIMEOUT
+        finally:
+            mc.set_debug(0, 1_000_000_000)
+        y = mc.moe_forward(x, g, shape, L.bits, packed, workspace=ws)
+        mc.check_status(ws)
+    finally:
+        mc.set_path(old)
+    torch.cuda.synchronize()
+    ref, *_ = oracle_layer(L, oracle_mats(L))
+    assert_close(y.float().cpu().numpy(), ref, "GEMM after an expired wait")
+
+
 def test_prefill_mixtral_shape(mc):
     """Mixtral-8x7b-shaped prefill layer, 4096 tokens with skewed expert loads
     (the prefill workload), outputs checked on the tokens of every expert's
