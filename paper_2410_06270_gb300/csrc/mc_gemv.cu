@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) gemv_kernel(ExpertParams p)
 constexpr int kPPKPS = 2;                  // 128-column steps per stage
 constexpr int kPPSlots = 2;                // ring slots per group
 constexpr int kPPThreads = 2 * (kCW + 1) * 32;
-constexpr int kPPMinPairs = 20;            // 2 T from which a quantised layer takes this kernel
+constexpr int kPPMinPairs = 32;            // 2 T from which a quantised layer takes this kernel
 
 struct PPGroup {
     uint64_t full[kPPSlots], empty[kPPSlots];
@@ -1093,10 +1093,15 @@ int launch_gemv(ExpertParams ep, cudaStream_t st)
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "device query: %s", cudaGetErrorString(err));
     // 16-bit experts are all or none of a layer (check_bits).  Quantised layers of
-    // >= 10 tokens run the two-group kernel.  Mixtral-8x7b layer, one group / two groups:
-    // 5 tokens 113.1 / 114.3 us, 8: 114.8 / 115.4, 9: 120.9 / 117.4, 12: 122.1 / 117.2, 15:
-    // 122.1 / 117.9 (with about one item per SM one group idles and the other's two-slot
-    // ring is too shallow to keep the stream busy: 1 token 58 / 65 us when it was measured)
+    // >= 16 tokens run the two-group kernel.  It is the faster one where every SM gets many
+    // items (16 tokens, all 8 experts of the Mixtral-8x7b layer: 132.5 / 125 us with one /
+    // two groups when it was made) and the slower one where few experts are touched, or a
+    // matrix has few row blocks: then one group idles while the other's two-slot ring is
+    // too shallow to keep the stream busy.  At 10 to 15 tokens which it is depends on how
+    // the tokens fall, which the host does not know, and it loses more than it gains:
+    // Mixtral-8x7b 12 tokens 118.8 / 115.3 us where an expert has over 8 pairs, 100.7 / 108.4
+    // where none has; 8x22b 12 tokens 190.8 / 201.5; H 2048, F 7168 15 tokens 48.8 / 50.4;
+    // H 4096, F 1024 12 tokens 31.0 / 42.3; 2 experts of H 2048, F 7168 29.5 / 38.2
     const bool dense = ep.bits[0] == 16;
     if (!dense && ep.Pmax >= kPPMinPairs) {
         const size_t smp = pp_smem(ep.group);
