@@ -398,11 +398,13 @@ __device__ __forceinline__ void permute_block(const PermuteParams &p)
     }
 }
 
-// The same placement for at most kPermKeys pairs per thread: every pair's key is loaded
+// The same placement for 2 to kPermKeys pairs per thread: every pair's key is loaded
 // once, all loads in flight together, the warps' counts of all passes go to shared
 // memory, and one scan per expert (a warp each) gives every (pass, warp) its start, so
 // that the placement needs three block barriers in all instead of five per pass: 4096
-// tokens 20 -> 13 us between events.
+// tokens 20 -> 13 us between events.  Up to one pair per thread permute_block's single
+// pass is the shorter one (mc_route, permute_keys / permute_block: 65 tokens 6.7 / 5.9 us,
+// 512: 7.7 / 6.9; two passes, 600 tokens: 7.9 / 8.2).
 constexpr int kPermKeys = 8;
 
 __device__ __forceinline__ void permute_keys(const PermuteParams &p)
@@ -571,7 +573,7 @@ __global__ void __launch_bounds__(1024) permute_kernel(PermuteParams p)
     pdl_trigger();
     pdl_wait();
     if (p.T <= kPermWarpMaxT) permute_warp(p);  // one warp
-    else if (2 * p.T <= kPermKeys * (int)blockDim.x) permute_keys(p);
+    else if (2 * p.T > (int)blockDim.x && 2 * p.T <= kPermKeys * (int)blockDim.x) permute_keys(p);
     else permute_block(p);
 }
 

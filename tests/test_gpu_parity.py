@@ -121,12 +121,12 @@ def test_single_launch_routing_places_like_the_two_launch_one(mc, T):
         mc.set_debug(0, 1_000_000_000)
 
 
-@pytest.mark.parametrize("T,H,E", [(152, 256, 8), (153, 4224, 8), (154, 256, 3), (515, 384, 9), (1023, 256, 5),
-                                   (4096, 128, 8), (4097, 128, 8)])
+@pytest.mark.parametrize("T,H,E", [(152, 256, 8), (153, 4224, 8), (154, 256, 3), (512, 256, 8), (515, 384, 9),
+                                   (1023, 256, 5), (4096, 128, 8), (4097, 128, 8)])
 def test_routing_of_many_tokens(mc, T, H, E):
     """The kernels for many tokens on both sides of their limits (153 tokens and 8
-    experts for several tokens per CTA, a ragged last group; 8192 pairs for the
-    one-load placement): bit-exact against the oracle, and weights bit for bit those of
+    experts for several tokens per CTA, a ragged last group; 1024 and 8192 pairs for
+    the one-load placement): bit-exact against the oracle, and weights bit for bit those of
     the same tokens routed a few at a time."""
     L = synth.make_layer(T, H, 128, E, 64, [2] * E, 700 + T, gate_std=0.15, mu=0.4, protect_frac=0.2, experts=False)
     _with_drops(L, T // 10, 701)
