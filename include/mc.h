@@ -317,6 +317,11 @@ int mc_set_debug(int flags, unsigned long long timeout_ns);
  * *status (device int32, may be NULL).  For the test suite; not on the layer path. */
 int mc_selftest_umma(const void *A, const void *B, float *D, int N, int K, int32_t *status, void *stream);
 
+/* Self-test of the layer's last launch without column splits (Eq. 1's sum over the two
+ * slots): y[t] = w[t][0] o[inv[2t]] + w[t][1] o[inv[2t+1]], a term with inv < 0 absent;
+ * o = opart, fp32 rows of H columns, y bf16 [T, H].  For the test suite. */
+int mc_selftest_combine(const float *opart, const float *w, const int32_t *inv, int T, int H, void *y, void *stream);
+
 /* Synchronise `stream`, read the status word at the start of `workspace`, clear
  * it, and return MC_OK or the recorded MC_ERR_* code. */
 int mc_check_status(void *workspace, void *stream);

@@ -71,6 +71,7 @@ def load():
         "mc_rmsnorm": (I, [P, P, I, I, F32, P, P]),
         "mc_add": (I, [P, P, Z, P, P]),
         "mc_selftest_umma": (I, [P, P, P, I, I, P, P]),
+        "mc_selftest_combine": (I, [P, P, P, I, I, P, P]),
         "mc_token_importance_workspace_size": (Z, [I]),
         "mc_token_importance": (I, [P, P, I, I, I, F32, P, P, P, Z, P]),
         "mc_odp_threshold_host": (I, [P, P, I, ctypes.c_double, P]),
@@ -481,5 +482,15 @@ def selftest_umma(A, B, status=None, a_in_tmem=False):
     n = -B.shape[0] if a_in_tmem else B.shape[0]
     _check(load().mc_selftest_umma(_ptr(A), _ptr(B), _ptr(D), n, A.shape[1], _ptr(status), _stream()))
     return D
+
+
+def selftest_combine(opart, w, inv):
+    """The layer's last launch: y[t] = w[t, 0] opart[inv[t, 0]] + w[t, 1] opart[inv[t, 1]]
+    (a term with inv < 0 absent) in bf16, for w fp32 [T, 2], inv int32 [T, 2]."""
+    import torch
+    T, H = w.shape[0], opart.shape[1]
+    y = torch.empty((T, H), dtype=torch.bfloat16, device=w.device)
+    _check(load().mc_selftest_combine(_ptr(opart), _ptr(w), _ptr(inv), T, H, _ptr(y), _stream()))
+    return y
 
 

@@ -995,12 +995,13 @@ __global__ void __launch_bounds__(256) combine1_kernel(CombineParams p)
 {
     pdl_trigger();
     pdl_wait();
-    const int H4 = p.H / 4;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= p.T * H4) return;
+    // (unsigned: T H / 4 reaches 2^31 where T H / 8 fits an int; launch_combine refuses 2^32)
+    const unsigned H4 = p.H / 4;
+    const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (unsigned)p.T * H4) return;
     const int t = idx / H4, c = (idx % H4) * 4;
-    const int2 q2 = *reinterpret_cast<const int2 *>(p.inv + 2 * t);
-    const float2 w2 = *reinterpret_cast<const float2 *>(p.w + 2 * t);
+    const int2 q2 = *reinterpret_cast<const int2 *>(p.inv + 2 * (size_t)t);
+    const float2 w2 = *reinterpret_cast<const float2 *>(p.w + 2 * (size_t)t);
     const uint2 rv = p.resid ? *reinterpret_cast<const uint2 *>(p.resid + (size_t)t * p.H + c) : make_uint2(0, 0);
     float4 a = make_float4(0, 0, 0, 0), b = a;
     if (q2.x >= 0) a = __ldcs(reinterpret_cast<const float4 *>(p.opart + (size_t)q2.x * p.H + c));
@@ -1161,15 +1162,14 @@ int launch_gemv(ExpertParams ep, cudaStream_t st)
 int launch_combine(const CombineParams &cp, cudaStream_t st)
 {
     if (cp.KS < 1 || cp.KS > kMaxKS) return set_error(MC_ERR_INVALID_ARG, "combine: %d column splits", cp.KS);
+    const size_t n = (size_t)cp.T * (cp.H / 4);  // threads
+    if (n > 0xffffff00ull) return set_error(MC_ERR_INVALID_ARG, "combine: T=%d, H=%d: %zu threads", cp.T, cp.H, n);
     profile_begin(kKCombine, st);
     cudaError_t err;
-    if (cp.KS > 1 || cp.T <= kCombine4MaxT) {
-        const int n = cp.T * (cp.H / 4);
-        err = launch_k(combine4_kernel, dim3((n + 127) / 128), dim3(128), 0, st, cp);
-    } else {
-        const int n = cp.T * (cp.H / 4);
-        err = launch_k(combine1_kernel, dim3((n + 255) / 256), dim3(256), 0, st, cp);
-    }
+    if (cp.KS > 1 || cp.T <= kCombine4MaxT)
+        err = launch_k(combine4_kernel, dim3((unsigned)((n + 127) / 128)), dim3(128), 0, st, cp);
+    else
+        err = launch_k(combine1_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, cp);
     profile_end(kKCombine, st);
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "combine launch: %s", cudaGetErrorString(err));
     return MC_OK;

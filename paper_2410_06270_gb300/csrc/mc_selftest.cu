@@ -1,8 +1,10 @@
 // mc_selftest.cu -- a one-CTA fp16 GEMM through the tcgen05 path (SW128 operands
 // written by threads, one-thread MMA issue, commit to an mbarrier, TMEM loads).
 // It checks the tensor-core building blocks of mc_umma.cuh against a plain
-// matrix product and is exported for the test suite only.
+// matrix product and is exported for the test suite only, like the combine's launch
+// on inputs of the test's own.
 #include "mc_host.h"
+#include "mc_kernels.h"
 #include "mc_umma.cuh"
 
 namespace mc {
@@ -151,4 +153,22 @@ extern "C" int mc_selftest_umma(const void *A, const void *B, float *D, int N, i
     err = cudaGetLastError();
     if (err != cudaSuccess) return set_error(MC_ERR_CUDA, "launch: %s", cudaGetErrorString(err));
     return MC_OK;
+}
+
+extern "C" int mc_selftest_combine(const float *opart, const float *w, const int32_t *inv, int T, int H, void *y,
+                                   void *stream)
+{
+    clear_error();
+    if (!opart || !w || !inv || !y) return set_error(MC_ERR_INVALID_ARG, "NULL pointer argument");
+    if (T <= 0 || H <= 0 || H % 128) return set_error(MC_ERR_INVALID_ARG, "need T > 0, H a positive multiple of 128");
+    CombineParams cp{};
+    cp.opart = opart;
+    cp.w = w;
+    cp.inv = inv;
+    cp.T = T;
+    cp.H = H;
+    cp.KS = 1;
+    cp.Pmax = 2 * T;
+    cp.y = (__nv_bfloat16 *)y;
+    return launch_combine(cp, (cudaStream_t)stream);
 }

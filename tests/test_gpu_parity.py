@@ -485,6 +485,23 @@ def test_activation_outside_fp16_range_is_reported(mc):
 
 # ------------------------------------------------------------- rmsnorm ----
 
+@pytest.mark.parametrize("T,H", [(65, 128), (1001, 4096), (131075, 65536)])
+def test_combine_of_any_size(mc, T, H):
+    """The last launch, up to outputs whose 4-column groups outnumber an int (2^33 values
+    and some).  Rows and weights are small multiples of powers of two, so that fp32 sums
+    and their bf16 roundings are exact."""
+    g = torch.Generator(device="cuda").manual_seed(T)
+    o = torch.randint(-8, 9, (5, H), generator=g, device="cuda").float()
+    w = torch.tensor([1.0, 0.5, 0.25], device="cuda")[torch.randint(0, 3, (T, 2), generator=g, device="cuda")]
+    inv = torch.randint(-1, 5, (T, 2), generator=g, device="cuda", dtype=torch.int32)
+    y = mc.selftest_combine(o, w, inv)
+    scale = torch.where(inv >= 0, w, torch.zeros_like(w))
+    for t0 in range(0, T, 4096):
+        q, s = inv[t0:t0 + 4096].clamp_min(0).long(), scale[t0:t0 + 4096]
+        want = s[:, :1] * o[q[:, 0]] + s[:, 1:] * o[q[:, 1]]
+        assert torch.equal(y[t0:t0 + 4096], want.bfloat16()), t0
+
+
 @pytest.mark.parametrize("H", [4096, 16384, 1001])
 def test_rmsnorm_and_add(mc, H):
     """RMSNorm against the oracle (16-byte rows up to H 16384 take the vector
