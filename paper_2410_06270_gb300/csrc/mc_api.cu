@@ -4,6 +4,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <vector>
 
@@ -38,10 +39,10 @@ static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Column splits of the W2 GEMV pass.  The workspace holds up to max_ks splits: the
 // kMaxKS of decode sizes have room of their own; from 65 tokens the partial outputs lie
-// over the GEMM's image buffers, which a GEMV call does not use, so the workspace is no
-// larger than the GEMM needs and one of more tokens serves every T.  The forward picks, among the divisors of F/128 that leave each
-// item at least two ring stages, the split count whose work items (estimated
-// chunks x 256-row block pairs x splits) fill the SMs' last wave best, the
+// over the GEMM's image buffers, which a GEMV call does not use, so that such a call needs
+// no more than the GEMM of as many tokens.  The forward picks, among the divisors of F/128
+// that leave each item at least two ring stages, the split count whose work items
+// (estimated chunks x 256-row block pairs x splits) fill the SMs' last wave best, the
 // smaller one on ties.  Above 64 tokens the chunk count depends on how the pairs fall,
 // so the most splits are taken: many short items leave a short last wave whatever it
 // is (Mixtral-8x7b layer, W2 launch without splits -> with 7: 65 tokens 112 -> 74 us,
@@ -152,6 +153,8 @@ static float neg_log_mu(float mu)
     return (float)(-log((double)mu));
 }
 
+size_t moe_workspace_need(const mc_shape *s, int T) { return carve(s, T, nullptr).total; }
+
 bool pdl_enabled() { return !(g_debug.load() & kDebugNoPdl); }
 int debug_flags() { return g_debug.load(); }
 uint64_t wait_bound_ns() { return g_timeout_ns.load(); }
@@ -184,7 +187,10 @@ int mc_set_debug(int flags, unsigned long long timeout_ns)
 size_t mc_moe_workspace_size(const mc_shape *shape, int T_max)
 {
     if (check_shape(shape) || T_max < 0) return 0;
-    return carve(shape, T_max, nullptr).total;
+    // A call of up to 64 tokens needs room for its column splits beside the images and may
+    // need more than one of 65 or some more; either kind needs more with more tokens.
+    const size_t most = moe_workspace_need(shape, T_max);
+    return T_max > 64 ? std::max(most, moe_workspace_need(shape, 64)) : most;
 }
 
 int mc_route(const void *x, const void *gate_w, int T, const mc_shape *shape, float mu, const uint8_t *protect,

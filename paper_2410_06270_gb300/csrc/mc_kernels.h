@@ -173,6 +173,8 @@ int moe_forward_ex(const void *x, const void *gate_w, int T, const mc_shape *sha
                    const void *packed_dev, float mu, const uint8_t *protect, void *y, const LayerPrePost *pp,
                    void *workspace, size_t ws_bytes, int32_t *topk_idx_out, float *topk_w_out, uint8_t *pruned_out,
                    void *stream);
+// Workspace bytes of a call with T tokens (mc_moe_workspace_size: of any call with up to T).
+size_t moe_workspace_need(const mc_shape *s, int T);
 // The test hooks of mc_set_debug: its flags and the bound on device waits.
 int debug_flags();
 uint64_t wait_bound_ns();

@@ -31,10 +31,10 @@ extern "C" int mc_stack_forward(void *h, int T, const mc_shape *shape, int layer
         return set_error(MC_ERR_INVALID_ARG, "NULL pointer argument");
     int rc = check_shape(shape);
     if (rc) return rc;
-    const size_t need = mc_stack_workspace_size(shape, T);
-    if (ws_bytes < need) return set_error(MC_ERR_INVALID_ARG, "workspace has %zu bytes, needs %zu", ws_bytes, need);
-    const size_t fw = align256(mc_moe_workspace_size(shape, T));
+    const size_t fw = align256(moe_workspace_need(shape, T));
     const size_t act = align256((size_t)T * shape->H * 2);
+    const size_t need = fw + 2 * act;
+    if (ws_bytes < need) return set_error(MC_ERR_INVALID_ARG, "workspace has %zu bytes, needs %zu", ws_bytes, need);
     void *xn = (uint8_t *)workspace + fw, *y = (uint8_t *)workspace + fw + act;
     // With 16-byte aligned rows the layer's routing launch computes its RMSNorm (bit
     // for bit mc_rmsnorm) into xn and routes on it, and its combine adds the layer

@@ -161,11 +161,13 @@ def test_workspace_size_grows_with_tokens(mc):
 
 @pytest.mark.parametrize("dims", [(8, 4096, 14336, 128), (8, 6144, 16384, 128), (2, 1024, 1024, 64), (4, 2048, 256, 64)])
 def test_workspace_of_more_tokens_covers_fewer(mc, dims):
-    """A workspace sized for any T_max >= 65 covers every T from 65 up to it, across the
-    limit between the GEMV with column splits and the GEMM."""
+    """A workspace sized for any T_max covers every T up to it, across the end of the
+    decode sizes (64 tokens) and the limit between the GEMV with column splits and the
+    GEMM; so does a stack's."""
     s = mc.Shape(*dims)
-    sizes = [mc.workspace_size(s, T) for T in range(65, 301)]
-    assert sizes == sorted(sizes)
+    for size in (mc.workspace_size, lambda s, T: mc.load().mc_stack_workspace_size(ctypes.byref(s), T)):
+        sizes = [size(s, T) for T in range(1, 301)]
+        assert sizes == sorted(sizes)
 
 
 def test_odp_threshold_host_matches_oracle():

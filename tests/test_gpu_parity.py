@@ -226,19 +226,22 @@ def test_forward_w2_column_splits(mc, T):
 
 @pytest.mark.parametrize("E,H,F", [(8, 512, 4096), (2, 4096, 2048)])
 def test_one_workspace_across_the_gemm_limit(mc, E, H, F):
-    """A workspace of 130 tokens (GEMM) serves 119, 65 and 100 tokens (W2 column splits,
-    whose partial outputs lie over the GEMM's images) and again 130, each bit for bit
-    as with a workspace of its own."""
+    """A workspace of 130 tokens (GEMM), of 100 and of 65 serves every smaller call: 119,
+    100 and 65 tokens (W2 column splits, whose partial outputs lie over the GEMM's
+    images), 64, 16 and 1 (splits beside them) and again 130, each bit for bit as with a
+    workspace of its own."""
     shape = mc.Shape(E, H, F, 128)
-    ws = mc.alloc_workspace(shape, 130)
-    for T in (119, 130, 65, 100, 130):
+    wss = {T: mc.alloc_workspace(shape, T) for T in (130, 100, 65)}
+    for T in (119, 130, 65, 64, 16, 1, 100, 130):
         L = synth.make_layer(T, H, F, E, 128, ([3, 2, 1, 3, 2, 2, 1, 3])[:E], 990 + T, gate_std=0.05)
         shape, packed = _pack(mc, L)
         x, g, p = to_dev(L)
-        y = mc.moe_forward(x, g, shape, L.bits, packed, L.mu, p, workspace=ws)
         y_own = mc.moe_forward(x, g, shape, L.bits, packed, L.mu, p)
-        mc.check_status(ws)
-        assert torch.equal(y, y_own), "T=%d" % T
+        for T_max, ws in wss.items():
+            if T <= T_max:
+                y = mc.moe_forward(x, g, shape, L.bits, packed, L.mu, p, workspace=ws)
+                mc.check_status(ws)
+                assert torch.equal(y, y_own), "T=%d of %d" % (T, T_max)
 
 
 def test_forward_fractional_zeros(mc):
