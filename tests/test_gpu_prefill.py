@@ -2,11 +2,14 @@
 128 pairs, A operand dequantised into tensor memory) against the CPU oracle:
 ragged token blocks, empty and overloaded experts, an odd number of W2 row
 blocks, both group sizes, fractional zeros, ODP with protected tokens, the
-automatic path switch, and the Mixtral-8x7b-shaped prefill layer on sampled
-tokens."""
+automatic path switch, many work items per CTA, the narrow and the wide geometry,
+expired waits, and the Mixtral-8x7b-shaped prefill layer on sampled tokens."""
+import dataclasses
+
 import numpy as np
 import pytest
 
+import oracle
 import synth
 from helpers import assert_close, boundary_tokens, condition_routing, flat, oracle_layer, oracle_mats, to_dev
 
@@ -14,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-PATH_GEMM = 2  # mc_set_path: the tcgen05 grouped GEMM
+PATH_GEMV, PATH_GEMM = 1, 2  # mc_set_path: the mma.sync GEMV, the tcgen05 grouped GEMM
 
 
 @pytest.fixture(scope="module")
@@ -117,6 +120,48 @@ def test_bounded_wait_reports_timeout_and_context_survives(mc):
     torch.cuda.synchronize()
     ref, *_ = oracle_layer(L, oracle_mats(L))
     assert_close(y.float().cpu().numpy(), ref, "GEMM after an expired wait")
+
+
+@pytest.mark.parametrize("T,H,F,E,group", [
+    (2560, 128, 8192, 8, 128),   # W1,W3 items of one column step, 64 per token block; lone W2 blocks
+    (300, 128, 16384, 16, 64),   # the same with token blocks of at most 64 pairs
+    (2300, 1408, 1024, 8, 64),   # W2: five block pairs and a lone block per token block
+    (2300, 1408, 1024, 8, 128),
+])
+def test_prefill_many_items_per_cta(mc, T, H, F, E, group):
+    """Several items per CTA in both launches, so that every ring and barrier goes round:
+    thousands of one-step W1,W3 items (the item ring's tight case), wide and narrow, and a
+    lone W2 block followed by another item.  The tokens at the edges of the experts'
+    token blocks against the oracle, all of them against the GEMV path."""
+    L = synth.make_layer(T, H, F, E, group, [1, 2, 3, 2] * (E // 4), 370 + T, gate_std=0.05)
+    condition_routing(L)
+    idx, _, pr = oracle.route(L.x_f32(), L.gate_f32(), 0.0)
+    pairs = np.diff(oracle.permute(idx, pr, E)[0])
+    assert (pairs.max() <= 64) == (T == 300)
+    tokens = boundary_tokens(L, blocks=(128,))
+    got = _run(mc, L, PATH_GEMM)
+    ref, *_ = oracle_layer(L, oracle_mats(L), tokens)
+    assert_close(got[tokens], ref, "GEMM T=%d H=%d F=%d g=%d" % (T, H, F, group))
+    assert_close(got, _run(mc, L, PATH_GEMV).astype(np.float64), "GEMM vs GEMV")
+
+
+def test_prefill_narrow_and_wide_agree(mc):
+    """The longest prefixes of a batch whose largest expert has 64 and 65 pairs: one takes
+    the narrow geometry (two accumulator sets), the other the wide one.  Both against the
+    oracle, and bit for bit the same on the tokens they share."""
+    L = synth.make_layer(300, 384, 2048, 8, 128, [3, 2, 1, 3, 2, 2, 1, 3], 380, gate_std=0.05)
+    condition_routing(L)
+    idx, *_ = oracle.route(L.x_f32(), L.gate_f32(), 0.0)
+    largest = np.stack([np.cumsum((idx == e).any(axis=1)) for e in range(L.E)]).max(axis=0)
+    out = []
+    for most in (64, 65):
+        T = int(np.searchsorted(largest, most, side="right"))
+        assert largest[T - 1] == most
+        P = dataclasses.replace(L, T=T, x=L.x[:T])
+        out.append(_run(mc, P, PATH_GEMM))
+        ref, *_ = oracle_layer(P, oracle_mats(P))
+        assert_close(out[-1], ref, "largest expert %d pairs" % most)
+    assert np.array_equal(out[1][:len(out[0])], out[0])
 
 
 def test_prefill_mixtral_shape(mc):
