@@ -19,8 +19,8 @@ constexpr int kPathAuto = 0, kPathGemv = 1, kPathGemm = 2;
 static std::atomic<int> g_path{kPathAuto};
 // pairs (2 T) from which mc_moe_forward's automatic choice is the prefill GEMM.
 // Mixtral-8x7b layer, GEMV (each weight tile decoded once per 16-pair chunk) / GEMM
-// (once per 128-pair token block): 32 tokens 149 / 195 us, 64: 214 / 199, 80: 257 /
-// 203, 96: 288 / 206, 119: 334 / 206, 128: 383 / 208.  The line lies above the
+// (once per 128-pair token block): 32 tokens 150 / 195 us, 64: 214 / 196, 80: 256 /
+// 201, 96: 289 / 203, 119: 334 / 203, 128: 381 / 204.  The line lies above the
 // crossover in time (~60 tokens) because the GEMM multiplies weights rounded to fp16
 // and the GEMV path exact codes: relative error of the layer output against 64 bits
 // 1.9e-3 and 1.7e-3.  A lower line would lose precision between the two.
@@ -45,9 +45,11 @@ static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // (estimated chunks x 256-row block pairs x splits) fill the SMs' last wave best, the
 // smaller one on ties.  Above 64 tokens the chunk count depends on how the pairs fall,
 // so the most splits are taken: many short items leave a short last wave whatever it
-// is (Mixtral-8x7b layer, W2 launch without splits -> with 7: 65 tokens 112 -> 74 us,
-// 80: 112 -> 88, 96: 112 -> 98, 112: 112 -> 103; the layer 252 -> 218, 279 -> 258, 300 ->
-// 289, 310 -> 305).
+// is (without splits / with 8, us, Mixtral-8x7b: W2 launch 65 tokens 115 / 75, 80: 115 / 88,
+// 96: 114 / 98, 112: 115 / 103, 119: 124 / 115; layer 254 / 216, 280 / 256, 301 / 288, 310 /
+// 303, 339 / 334, on other draws of 119 tokens 326 / 328 and 327 / 331; layers of 8x22b 580 /
+// 540 at 119 tokens, of H 2048, F 7168 106 / 73 at 65 and 126 / 102 at 119, of 2 experts of
+// that size 98 / 66 at 65).
 
 static size_t image_bytes(const mc_shape *s, int T)
 {

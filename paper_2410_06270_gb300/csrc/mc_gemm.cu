@@ -30,12 +30,12 @@
 // What sets the pace.  The tensor pipe takes 1026 cycles for a step's 16 MMAs at
 // N = 128 and 515 at N = 64, whatever copies, tensor-memory stores and shared-memory
 // loads run beside it; the conversion alone takes ~51 cycles per 16x128 tile and SM
-// (820 a step) with 8 warps as with 16: its LOP3, HADD2 and HFMA2 each issue every
-// other cycle.  What kept the MMAs from either pace was their issue: from a
-// `lane == 0` branch 8 MMAs take 541 cycles of moves into uniform registers, and 859
-// beside 16 busy warps (elect_one).  Mixtral-8x7b layer, W1,W3 / W2 launch: 256 tokens
-// (N ~ 60) 157 / 99 -> 135 / 78 us, 4096 tokens 1424 / 755 -> 1298 / 646 us (1.49
-// PFLOP/s, 0.85 of the sustained cuBLAS rate; power-capped).
+// (820 a step) with 8 warps as with 16: a probe's lop3, __hsub2 and __hfma2 each issue
+// every other cycle.  What kept the MMAs from either pace was their issue: under
+// `lane == 0` 8 MMAs take 541 cycles, and 859 beside 16 busy warps (elect_one).
+// Mixtral-8x7b layer, W1,W3 / W2 launch: 256 tokens (N ~ 60) 157 / 99 -> 131 / 76 us,
+// 4096 tokens 1424 / 755 -> 1316 / 657 us (1.46 PFLOP/s, 0.83 of the sustained cuBLAS
+// rate; power-capped: 1298 / 646 in another run).
 // Tensor memory (512 columns): accumulators of streams 0/1 at columns 0 / 128 (when
 // every token block has <= 64 pairs, two accumulator sets of 64 columns each, so
 // that an item's epilogue overlaps the next item's MMAs), each stream's two A
@@ -68,7 +68,10 @@ static_assert(kGItemRing >= kGMaxW + 4 + 3, "item ring");
 
 // Ring geometry of a call: the weight slots hold a 3-bit step of both streams, the
 // image slots 128 or (narrow) 64 rows; what is left beside the h staging is split so
-// that either ring covers a copy's latency.
+// that either ring covers a copy's latency (4 image and 5 weight slots, 4 of them at group
+// 64; narrow 6 and 8).  One expert of more than 64 pairs makes the whole call wide, which
+// costs 1 %: the Mixtral-8x7b layer narrow / forced wide at 200 tokens 211.5 / 213.7 us, at
+// 256 with ODP 217.3 / 219.4.
 struct GGeom {
     int atom;               // bytes between an image slot's two 64-column atoms
     int wslot, nw, ni;      // weight slot bytes, weight and image slots
@@ -320,8 +323,8 @@ __device__ __forceinline__ void tmem_st_16x256_x8(uint32_t taddr, const uint32_t
 
 // A step's two tiles of one converter warp: converted and stored, the first store
 // after the MMAs have read the buffer.  One code path per width from the packed words
-// to the store: tcgen05.st takes 32 consecutive registers, and a store shared by the
-// widths' branches costs a move per register.  False once the CTA aborted.
+// to the store (a store behind the widths' branches, shared by them: the ODP layer at
+// 256 tokens 241 -> 245 us).  False once the CTA aborted.
 template <int BITS, int GPT>
 __device__ __forceinline__ bool convert_store(const RawTile<GPT> &ta, const RawTile<GPT> &tb, uint32_t abuf, bool wait,
                                               uint64_t *aempty, uint32_t parity, const ExpertParams &p, GShared *sh)

@@ -987,9 +987,9 @@ __global__ void __launch_bounds__(kPPThreads, 1) gemv_pp_kernel(ExpertParams p)
 // with a residual (the pre-norm stack), y[t] = resid[t] + that, rounded to bf16
 // first (the layer's own output) and once more after the fp32 add.
 //
-// A single split (the GEMM, and the GEMV above 64 tokens when it takes one): both slots' rows loaded
-// at once, 4 columns per thread, no per-split registers, so that enough loads are in
-// flight to stream the partial outputs: 71 -> 30 us between events at 4096 tokens (134
+// A single split (the GEMM, and the GEMV above 64 tokens when it takes one): both slots'
+// rows loaded at once, 4 columns per thread, no per-split registers, so that enough loads
+// are in flight to stream the partial outputs: 71 -> 30 us between events at 4096 tokens (134
 // MB in, 33 MB out; 8 columns per thread, slot by slot, before).
 __global__ void __launch_bounds__(256) combine1_kernel(CombineParams p)
 {

@@ -154,8 +154,9 @@ int launch_combine(const CombineParams &cp, cudaStream_t st);
 int max_chunks_for(int T, int E);
 int32_t *route_done_word();  // mc_route's arrival word for the single-launch routing
 // Column splits of the W2 GEMV pass: the most a workspace for T tokens holds, and
-// the count a forward picks (the one whose work items fill the SMs' last wave
-// best, among the divisors of F/128 that leave every item >= 8 column steps).
+// the count a forward picks among the divisors of F/128 that leave every item >= 8
+// column steps (up to 64 tokens the one whose work items fill the SMs' last wave best,
+// above them the most that fit).
 int max_ks(const mc_shape *s, int T);
 int choose_ks(const mc_shape *s, int T, int nsm);
 // The pre-norm residual form of one layer, for mc_stack_forward: with norm_in,

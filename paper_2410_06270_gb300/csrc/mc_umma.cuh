@@ -95,11 +95,10 @@ __device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         : "memory");
 }
 
-// True in one lane of the (converged) warp, the same one every time.  MMAs issued
-// under `if (elect_one())` in warp-uniform code take their operands from uniform
-// registers; under `if (lane == 0)` every operand is moved there first, instruction
-// by instruction: 8 issues took 541 cycles alone and 859 beside 16 busy warps, with
-// the elected lane and descriptors formed by adding constants 160 and 249.
+// True in one lane of the (converged) warp, the same one every time.  The form of the
+// branch sets what an MMA's issue costs: 8 issues under `if (lane == 0)` took 541 cycles
+// alone and 859 beside 16 busy warps, under `if (elect_one())` in warp-uniform code
+// with descriptors formed by adding constants 160 and 249 (probe kernels).
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t ok;
